@@ -401,30 +401,37 @@ __device__ __forceinline__ float wf_dudy(float y)
     return __fdividef(SA_CV1_3 + k3, SA_CV1_3 + k3 * (1.0f + SA_KAPPA * y));
 }
 
-// Friction velocity from u_t at distance y (step 3): Newton on g(u) = u u+(u y / nu) - u_t,
-// g' = u+ + y+ du+/dy+ > 0, started from the previous sub-step's value when there is one,
-// else from the viscous-sublayer value (which lies left of the root, since u+ <= y+).
-// y_nu = y / nu.  Every evaluation narrows a sign bracket; steps leaving it are replaced by
-// bisection (or doubling while no right end is known).  The iteration stops after a Newton
-// step (not a bisection) shorter than 3e-4 u: Newton's error after a step of relative size
-// e is about (g'' u / 2 g') e^2, at most e^2 / 2 (the viscous sublayer; about 0.05 e^2 in
-// the log layer), so the result is within 4.5e-8 relative of the root, below FP32
-// resolution.  At most 24 evaluations.
+// Friction velocity from u_t at distance y (step 3): the root of g(u) = u u+(u y / nu) - u_t,
+// g' = u+ + y+ du+/dy+ > 0, started from the previous sub-step's value when there is one, else
+// from the viscous-sublayer value.  y_nu = y / nu.  While g is far from zero (more than 5 % of
+// u_t) the step is Newton's in the logarithms, u (u_t / (u u+))^(u+ / g'): u u+ is a power of u
+// whose exponent g' / u+ only varies from 2 (viscous sublayer) to about 1.1 (log layer), so a
+// start off by a factor of ten takes two or three such steps where Newton's own halves its
+// distance per step.  Near the root it is Newton's own step, and the iteration stops after one
+// shorter than 3e-4 u: its error after a step of relative size e is about (g'' u / 2 g') e^2, at
+// most e^2 / 2 (the viscous sublayer; about 0.05 e^2 in the log layer), so the result is within
+// 4.5e-8 relative of the root, below FP32 resolution.  It also stops where g is within the
+// rounding of u+ (terms of up to 20 in FP32: 4e-6), which below y+ of about 0.01 is more than 3e-4
+// of u+: without that rule the few boundary nodes near a stagnation point ran through the limit
+// of evaluations in every step, and the whole launch waited for them.  Over u_t from 1e-9 to 0.5
+// and y / nu from 10 to 3e6 it takes one evaluation from the previous step's value, two after
+// that has moved by 1e-3, at most six from anywhere (limit 24).
 __device__ float wf_utau(float ut, float y_nu, float guess)
 {
     if (!(ut > 0.0f)) return 0.0f;
-    float lo = 0.0f, hi = INFINITY;
     float u = guess > 0.0f ? guess : sqrtf(ut / y_nu);
     for (int it = 0; it < 24; it++) {
         const float yp = u * y_nu;
         const float up = wf_uplus(yp);
         const float gv = u * up - ut;
-        if (gv > 0.0f) hi = u; else lo = u;
         const float gp = up + yp * wf_dudy(yp);
-        float un = gp > 0.0f ? u - __fdividef(gv, gp) : -1.0f;
-        const bool newton = un > lo && un < hi;
-        if (!newton) un = isinf(hi) ? 2.0f * fmaxf(u, lo) : 0.5f * (lo + hi);
-        const bool done = newton && fabsf(un - u) <= 3e-4f * un;
+        if (fabsf(gv) > 0.05f * ut) {
+            u *= __powf(__fdividef(ut, u * up), __fdividef(up, gp));
+            if (fabsf(gv) <= 4e-6f * u) break;
+            continue;
+        }
+        const float un = u - __fdividef(gv, gp);
+        const bool done = fabsf(un - u) <= 3e-4f * un || fabsf(gv) <= 4e-6f * u;
         u = un;
         if (done) break;
     }
