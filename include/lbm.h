@@ -92,7 +92,7 @@ typedef struct {
                                      word, chi, rho and u; with SA-neg also chi written, u and 1/d^2 read) */
     double device_bytes;          /* device memory held by the handle                                */
     long long work_tiles[16];     /* tiles per level holding an active or ghost fluid cell           */
-    long long work_warps[16];     /* 16 x 2-cell warps of those tiles that hold one (LBM_SCHED_WARPS) */
+    long long work_warps[16];     /* 16 x 2-cell warps of those tiles that hold one                   */
 } lbm_info;
 
 /* Per-kernel-class timing of eagerly launched steps (CUDA events on the solver stream). */
@@ -280,26 +280,26 @@ lbm_status lbm_get_info(lbm_solver *s, lbm_info *out);
  * the solver stream; accumulate device time per kernel class.  Same results as lbm_step. */
 lbm_status lbm_time_kernels(lbm_solver *s, int n_coarse_steps, lbm_kernel_times *out);
 
-/* Grid schedules of the fused level kernel (lbm_autotune, lbm_set_launch_variant). */
-#define LBM_SCHED_TILE 0      /* one 256-thread block per work tile                              */
-#define LBM_SCHED_PERSIST 1   /* a grid of 2 x SMs x budget blocks striding over the work tiles  */
-#define LBM_SCHED_WARPS 2     /* two-warp blocks over the list of work warps (16 x 2 cells each
-                                 of a work tile that hold an active or ghost fluid cell; shape 0),
-                                 ordered warps with boundary nodes, with band or coalescing cells,
-                                 with other active cells, with ghosts only                      */
-#define LBM_SCHED_WARPS4 3    /* four-warp blocks over the same list (shape 0)                    */
+/* Grid schedules of the fused level kernel (lbm_autotune, lbm_set_launch_variant).  Every
+ * launch goes over the level's work warps (16 x 2 cells each of a work tile that hold an
+ * active or ghost fluid cell), those with boundary nodes first, then with band or coalescing
+ * cells, with other active cells, with ghosts only, and last the plain ones (active cells
+ * away from walls, interfaces and box edges); the schedule gives the warps of a block. */
+#define LBM_SCHED_TILE 0      /* four-warp blocks                                                 */
+#define LBM_SCHED_PERSIST 1   /* the same                                                         */
+#define LBM_SCHED_WARPS 2     /* two-warp blocks                                                  */
+#define LBM_SCHED_WARPS4 3    /* four-warp blocks                                                 */
 
 /* Launch autotuner.  Not part of the paper's method (Sec 2.1 gives the level schedule, not
  * its mapping to a GPU).  For each level it picks one of LBM_TUNE_CANDIDATES launch forms
- * of the fused level kernel: a register budget of at most 48 or 40 registers a thread (at
- * least 5 or 6 resident 256-thread blocks per SM), each with one of the grid schedules
- * LBM_SCHED_* and, for the tile schedules, one of two work shapes of a warp within the
- * 32 x 8 cell tile (shape 0: a 16 x 2 block of cells; shape 1: a 32-cell row, whose
- * accesses shifted by one cell touch fewer sectors and whose restriction goes through
- * shared memory).  The choice comes from per-launch CUDA-event timings of `steps` eager
+ * of the fused level kernel: one of the grid schedules LBM_SCHED_*, with min_blocks (5 or 6)
+ * and shape (0 or 1), which have no effect (the registers of a launch and the cells a lane
+ * takes follow from the level's size and kind) and stay in the report and in
+ * lbm_set_launch_variant for callers that hold saved variants.
+ * The choice comes from per-launch CUDA-event timings of `steps` eager
  * coarse steps per candidate, and is kept only if `steps` coarse steps through the step
- * graphs confirm it (against the same choice with one block per tile where it picked a
- * persistent grid, against the form before tuning, and against each candidate on every
+ * graphs confirm it (against the same choice with LBM_SCHED_TILE where it picked
+ * LBM_SCHED_PERSIST, against the form before tuning, and against each candidate on every
  * level; the fastest of these is kept), since launches overlap inside the
  * graphs.  Then it picks whether launches use programmatic dependent launch, from the time
  * of `steps` coarse steps through the step graphs each way, and recaptures the graphs with
@@ -314,11 +314,11 @@ typedef struct {
     int candidate_sched[LBM_TUNE_CANDIDATES];
     int candidate_shape[LBM_TUNE_CANDIDATES];
     double level_us[LBM_TUNE_CANDIDATES][16]; /* mean launch time of level l's kernel per candidate */
-    int min_blocks[16];                       /* chosen register budget per level                  */
+    int min_blocks[16];                       /* chosen min_blocks per level                       */
     int sched[16];                            /* chosen grid schedule per level (LBM_SCHED_*)      */
     int shape[16];                            /* chosen work shape per level                       */
     double step_us_confirm[3 + LBM_TUNE_CANDIDATES]; /* coarse step: per-level pick, pick with
-                                                 tile blocks for persistent grids, form before
+                                                 TILE for PERSIST, form before
                                                  tuning, then each candidate on every level    */
     int confirm_choice;                       /* index into step_us_confirm of the form kept    */
     double default_step_us;                   /* coarse step through the graphs before tuning      */
@@ -351,7 +351,8 @@ lbm_status lbm_set_state(lbm_solver *s, const void *buf, size_t size);
 lbm_status lbm_set_launch_variant(lbm_solver *s, const int *min_blocks, const int *sched, const int *shape,
                                   int pdl);
 
-/* The level kernel's work lists of a level, in launch order (also on host-only handles):
+/* The level kernel's work lists of a level in cost order (also on host-only handles; a launch
+ * takes the warps in this order, except that plain ones, of active cells only, come last):
  * warps 0 gives the work tiles (tiles holding an active or ghost fluid cell), warps 1 the
  * work warps (the 16 x 2-cell warps w of those tiles, cells x in [16 (w & 1), +16), y in
  * {2 (w >> 1), +1} of the tile, that hold one); both ordered by cost class (a boundary node

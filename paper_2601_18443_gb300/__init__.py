@@ -459,7 +459,7 @@ class Solver:
                     work_tiles=list(out.work_tiles[:L]), work_warps=list(out.work_warps[:L]))
 
     def autotune(self, steps=10):
-        """lbm_autotune: per-level register budget and PDL choice by timing; advances the
+        """lbm_autotune: per-level launch form and PDL choice by timing; advances the
         solve by the returned steps_taken coarse steps."""
         out = lbm_tune_report()
         self._check(self._lib.lbm_autotune(self._h, int(steps), C.byref(out)))
@@ -479,9 +479,9 @@ class Solver:
         self._check(self._lib.lbm_set_state(self._h, b.ctypes.data_as(C.c_void_p), b.size))
 
     def set_launch_variant(self, min_blocks, pdl=1, sched=None, shape=None):
-        """lbm_set_launch_variant: per-level register budget (5 or 6 blocks per SM), grid
-        schedule (SCHED_TILE, SCHED_PERSIST, SCHED_WARPS or SCHED_WARPS4), work shape of a warp
-        (0 a 16 x 2 block, 1 a 32-cell row; 0 with the warp-list schedules) and PDL."""
+        """lbm_set_launch_variant: per level the grid schedule (SCHED_*: the warps of a block),
+        min_blocks (5 or 6) and shape (0 or 1; 0 with the warp-list schedules), which have no
+        effect, and PDL."""
         mb = np.ascontiguousarray(min_blocks, dtype=np.int32)
         pe = np.ascontiguousarray(sched if sched is not None else [SCHED_TILE] * len(mb), dtype=np.int32)
         sh = np.ascontiguousarray(shape if shape is not None else [0] * len(mb), dtype=np.int32)

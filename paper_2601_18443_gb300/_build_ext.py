@@ -41,17 +41,14 @@ def build(force: bool = False, verbose: bool = False, bounds_check: bool = False
     os.makedirs(OUT_DIR, exist_ok=True)
     nvcc = _nvcc()
     tag = f".{os.getpid()}" + (".check" if bounds_check else "")
-    objs = {name: os.path.join(OUT_DIR, name.rsplit(".", 1)[0] + tag + ".o")
-            for name in ("grid.cpp", "kernels.cu", "lbm_capi.cu", "noalloc.cu")}
+    cus = ("level_f32.cu", "level_f16.cu", "level_bf16.cu", "kernels.cu", "lbm_capi.cu", "noalloc.cu")
+    objs = {name: os.path.join(OUT_DIR, name.rsplit(".", 1)[0] + tag + ".o") for name in ("grid.cpp",) + cus}
     cuflags = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-fopenmp",
                "-Xptxas", "-v" if verbose else "-O3"] + ARCH + (["-DLBM_BOUNDS_CHECK"] if bounds_check else [])
     cmds = [
         ["g++", "-O3", "-std=c++17", "-fPIC", "-fopenmp", "-ffp-contract=off", "-c",
          os.path.join(CSRC, "grid.cpp"), "-o", objs["grid.cpp"]],
-        [nvcc] + cuflags + ["-c", os.path.join(CSRC, "kernels.cu"), "-o", objs["kernels.cu"]],
-        [nvcc] + cuflags + ["-c", os.path.join(CSRC, "lbm_capi.cu"), "-o", objs["lbm_capi.cu"]],
-        [nvcc] + cuflags + ["-c", os.path.join(CSRC, "noalloc.cu"), "-o", objs["noalloc.cu"]],
-    ]
+    ] + [[nvcc] + cuflags + ["-c", os.path.join(CSRC, name), "-o", objs[name]] for name in cus]
     procs = [subprocess.Popen(c, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True) for c in cmds]
     logs = []
     for c, p in zip(cmds, procs):

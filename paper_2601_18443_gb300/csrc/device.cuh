@@ -21,12 +21,10 @@ struct LevelView {
     const int *parent;            // tile of level l-1 holding the parents, or -1
     const int *band_tiles;        // tiles with band cells
     int n_band_tiles;
-    const int *work_tiles;        // tiles with active or ghost fluid cells (the level kernel's grid),
-                                  // those with boundary nodes first, then with band or coalescing
-                                  // cells, then other active cells, then ghosts only
-    int n_work_tiles;
-    const int *work_warps;        // tile * 8 + w for each warp w (work shape 0) of a work tile that
-    int n_work_warps;             // holds an active or ghost fluid cell (the warp-list schedule)
+    const int *work;              // tile * 8 + w of the 16 x 2-cell warps w that hold an active or ghost
+    int n_gen_warps, n_pair_warps;// fluid cell: n_gen_warps entries in cost order, of which the first
+                                  // n_pair_warps / 2 blocks (with boundary nodes) stand twice, then
+    int n_plain;                  // n_plain (even) of plain active cells only (plain_warp)
     const uint32_t *flags;        // per slot
     const float *inv_d2;          // 1 / d^2, d the wall distance in level lattice units (SA-neg)
     const int *aux;               // per slot: wall record of a B node (finest level), band index of a
@@ -60,8 +58,6 @@ struct RecView {
     float *fpost;                 // 9 per record: post-collision f - w of the boundary node, last step
     const uint32_t *nfluid;       // per record: bit q set where the node B + c_q is active fluid
                                   // (present and not solid), for eq 27's interpolation
-    const float *yc;              // 18 per record: 1 / (1 + q_c) and q_c / (1 + q_c) per direction
-                                  // (eq 27's interpolation weights)
 };
 
 struct StepConsts {
@@ -95,26 +91,18 @@ struct LevelStep {
     int wall;           // this level holds the wall records (finest level)
     int restrict_up;    // write the restriction of this level's new fields into level l-1
     int pp;             // time level of level l-1 (restriction writes [pp ^ 1])
-    int shape;          // cells of a warp: 0 a 16 x 2 block, 1 a 32 x 1 row of the tile
     int *status;        // device status word (LBM_STATUS_* bits)
     unsigned long long *tl;  // launch timeline (lbm_set_timeline): 3 clock readings a block from
     int tl_base;             // record tl_base + blockIdx.x, or null
 };
 
-// Launch variant of a level's kernels (chosen by lbm_autotune): the register budget of the
-// fused level kernel, as the minimum resident blocks per SM (5 or 6), whether its blocks
-// persist over several tiles, the cells a warp covers within the tile, and whether
-// launches use programmatic dependent launch.  Every variant computes the same numbers
-// up to FP32 rounding.
+// Launch variant of a level's kernels (lbm_set_launch_variant, lbm_autotune): the warps of a
+// block, and whether launches use programmatic dependent launch.
 struct LevelTune {
-    int min_blocks;
+    int warps_per_block;   // 2 or 4
     int pdl;
-    int sched;          // LBM_SCHED_TILE: one block per work tile; LBM_SCHED_PERSIST: a grid of
-                        // 2 x SMs x min_blocks blocks striding over the work tiles;
-                        // LBM_SCHED_WARPS: two-warp blocks over the work-warp list (shape 0)
-    int shape;          // work shape of a warp (LevelStep::shape)
+    bool plain;            // plain blocks two to a warp (plain_warp)
 };
-
 
 // launchers (kernels.cu); all enqueue on the given stream
 void launch_level(cudaStream_t st, const LevelView &P, const LevelView *F, const LevelView *C, const RecView &R,
@@ -149,6 +137,7 @@ struct SolveDesc {
 };
 struct BatchArgs {
     int n;               // solves in this launch
+    bool plain;          // as LevelTune::plain
     SolveDesc d[LBM_BATCH_MAX];
 };
 struct ProlongDesc {

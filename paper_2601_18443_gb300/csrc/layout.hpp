@@ -13,6 +13,7 @@
 #define LBM_TY 8
 #define LBM_TILE (LBM_TX * LBM_TY)
 #define LBM_MAXL 16
+#define LBM_BLOCK 128            // most threads of a block of the level kernel
 
 // cell kinds
 #define KIND_ABSENT 0u

@@ -98,7 +98,7 @@ struct lbm_solver {
     LoadsView segs;
     StepConsts k;
     int parity[LBM_MAXL];
-    int min_blocks[LBM_MAXL];     // register budget of each level's kernel (lbm_autotune)
+    int min_blocks[LBM_MAXL];     // accepted and reported, without effect
     // prolongations of consecutive levels that read nothing the other writes go out as one
     // launch: prolong_indep[l] holds when no band cell of level l has a ghost of level l in
     // its 3 x 3 neighbourhood (prolongation l - 1 writes those ghosts, prolongation l reads
@@ -120,7 +120,7 @@ struct lbm_solver {
     unsigned pend_grid = 0;
     int pend_level = 0;
     int sched[LBM_MAXL];          // grid schedule (LBM_SCHED_*) of each level's kernel (lbm_autotune)
-    int shape[LBM_MAXL];          // work shape of a warp for each level's kernel (lbm_autotune)
+    int shape[LBM_MAXL];          // accepted and reported, without effect
     int pdl = 1;                  // programmatic dependent launch (lbm_autotune)
     bool off_schedule = false;    // single launches (lbm_step_launch) left the level schedule
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -318,6 +318,18 @@ static void flush_prolong(lbm_solver *s, cudaStream_t st, long long &nk)
     s->pend_grid = 0;
 }
 
+// Whether a launch over `warps` work warps takes the plain ones two to a warp.  Up to one wave of
+// resident warps (5 blocks of 4 a SM) a launch is one warp's latency, and a warp of one block is
+// the shorter one: 2700 work warps took 4.7 / 5.4 us (even / odd step, the 7-level polar request's
+// finest level) against 5.5 / 6.7 as pairs, 1400 warps 3.0 / 3.8 against 4.8 / 6.0.  Beyond that the
+// work per warp counts: 3100 warps (level 2 of the c/4096 workload) 5.3 / 6.4 us as pairs and
+// 5.4 / 6.3 one by one, 5000 (level 3) 5.5 / 6.3 and 7.6 / 8.4, 8800 (level 4) 8.2 / 10.2 and
+// 11.5 / 13.1.
+static bool plain_form(long warps, int sms) { return warps > 20 * (long)sms; }
+
+// warps of a block of the level kernel under a grid schedule
+static int block_warps(int sched) { return sched == LBM_SCHED_WARPS ? 2 : LBM_BLOCK / 32; }
+
 // One level-l step (Sec 2.1 recursive sub-cycling): the ghost fields of level l+1 are
 // reconstructed from level l at time t, level l+1 takes two sub-steps (the second one
 // restricts its new fields into the covered cells of level l), then one fused launch
@@ -352,18 +364,17 @@ static void advance(lbm_solver *s, cudaStream_t st, int l, int restrict_up, long
     ls.wall = (l == L - 1) && s->rec.n > 0;
     ls.restrict_up = restrict_up && C != nullptr;
     ls.pp = C ? s->parity[l - 1] : 0;
-    ls.shape = s->shape[l];
     ls.status = s->d_status;
     char nm[48];
     snprintf(nm, sizeof nm, "level %d %s step", l, ls.p ? "odd" : "even");
     NvtxRange range(s->tl_graph < 0 ? nm : "capture");
     {
-        const int base = tl_reserve(s, l, ls.p, std::max(P.n_work_tiles, (P.n_work_warps + 1) / 2));
+        const int base = tl_reserve(s, l, ls.p, (P.n_gen_warps + P.n_plain + 1) / 2);
         ls.tl = base >= 0 ? s->d_tl : nullptr;
         ls.tl_base = base;
     }
     mark_begin(s);
-    const lbmdev::LevelTune tu{s->min_blocks[l], s->pdl, s->sched[l], s->shape[l]};
+    const lbmdev::LevelTune tu{block_warps(s->sched[l]), s->pdl, plain_form(P.n_gen_warps + P.n_plain, s->k.sms)};
     lbmdev::launch_level(st, P, F, C, s->rec, s->k, ls, tu);
     mark_end(s, l == L - 1 ? KC_LEVEL_FINEST : KC_LEVEL_COARSE, P.ns, l);
     nk++;
@@ -703,8 +714,6 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
             for (int k = 3; k >= 0; k--)
                 for (long m = 0; m < nwt; m++)
                     if (tcls[m] == k) wt.push_back(G.work_tiles[m]);
-            v.work_tiles = upload(s, wt, ok);
-            v.n_work_tiles = (int)wt.size();
             H.work_tiles = wt;
         }
         {
@@ -737,9 +746,47 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
             for (int k = 3; k >= 0; k--)
                 for (long mw = 0; mw < nwt8; mw++)
                     if (wcls[mw] == k) ww.push_back(G.work_tiles[mw >> 3] * 8 + (int)(mw & 7));
-            v.work_warps = upload(s, ww, ok);
-            v.n_work_warps = (int)ww.size();
             H.work_warps = ww;
+            // the device's list: plain warps (every cell active fluid without any special bit, and
+            // every neighbour tile of the block present), an even number of them, after the others
+            const long nw = (long)ww.size();
+            std::vector<uint8_t> plain(nw, 0), has_bnode(nw, 0);
+#pragma omp parallel for schedule(static)
+            for (long m = 0; m < nw; m++) {
+                const int t = ww[m] >> 3, w = ww[m] & 7;
+                bool ok_w = true;
+                for (int c = 0; ok_w && c < 32; c++) {
+                    const int lx = (w & 1) * 16 + (c & 15), ly = (w >> 1) * 2 + (c >> 4);
+                    ok_w = H.flags[(size_t)t * LBM_TILE + ly * LBM_TX + lx] == KIND_ACTIVE;
+                    for (int d = 1; ok_w && d < 9; d++) {
+                        const int ax = lx + CXh[d], ay = ly + CYh[d];
+                        const int sx = ax < 0 ? -1 : (ax >= LBM_TX ? 1 : 0), sy = ay < 0 ? -1 : (ay >= LBM_TY ? 1 : 0);
+                        for (int e = 1; e < 9; e++)
+                            if (CXh[e] == sx && CYh[e] == sy && G.nbr[(size_t)t * 9 + e] < 0) ok_w = false;
+                    }
+                }
+                plain[m] = ok_w;
+                for (int c = 0; c < 32; c++) {
+                    const int lx = (w & 1) * 16 + (c & 15), ly = (w >> 1) * 2 + (c >> 4);
+                    const uint32_t f = H.flags[(size_t)t * LBM_TILE + ly * LBM_TX + lx];
+                    if ((f & (FL_KIND_MASK | FL_SOLID | FL_BNODE)) == (KIND_ACTIVE | FL_BNODE)) has_bnode[m] = 1;
+                }
+            }
+            std::vector<int> gw, pw;
+            for (long m = 0; m < nw; m++)
+                if (plain[m]) pw.push_back(ww[m]);
+            pw.resize(pw.size() & ~(size_t)1);
+            size_t left = pw.size();
+            v.n_pair_warps = 0;
+            for (long m = 0; m < nw; m++) {
+                if (plain[m] && left > 0) { left--; continue; }
+                gw.push_back(ww[m]);
+                if (l == L - 1 && has_bnode[m]) { gw.push_back(ww[m]); v.n_pair_warps += 2; }
+            }
+            v.n_gen_warps = (int)gw.size();
+            v.n_plain = (int)pw.size();
+            gw.insert(gw.end(), pw.begin(), pw.end());
+            v.work = upload(s, gw, ok);
         }
         v.flags = upload(s, H.flags, ok);
         v.inv_d2 = upload(s, inv_d2, ok);
@@ -767,7 +814,6 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         const lbmgrid::Level &G = s->g.lv[L - 1];
         std::vector<int> bslot(nr), nsv(nr), st_slot((size_t)nr * 16, -1), loop(nr);
         std::vector<float> st_wr((size_t)nr * 16, 0.f), st_wu((size_t)nr * 16, 0.f), nx(nr), ny(nr), dwb(nr), q((size_t)nr * 9, 0.f);
-        std::vector<float> yc((size_t)nr * 18, 0.f);
         for (int r = 0; r < nr; r++) {
             const lbmgrid::Record &R = s->g.recs[r];
             bslot[r] = (int)G.slot(R.i, R.j);
@@ -781,11 +827,7 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
                 st_wu[(size_t)r * 16 + m] = m < R.ns ? (float)wu[m] : 0.f;
             }
             nx[r] = (float)R.n[0]; ny[r] = (float)R.n[1]; dwb[r] = (float)R.dwb;
-            for (int d = 0; d < 9; d++) {
-                q[(size_t)r * 9 + d] = (float)R.q[d];
-                yc[(size_t)r * 18 + 2 * d] = (float)(1.0 / (1.0 + R.q[d]));
-                yc[(size_t)r * 18 + 2 * d + 1] = (float)(R.q[d] / (1.0 + R.q[d]));
-            }
+            for (int d = 0; d < 9; d++) q[(size_t)r * 9 + d] = (float)R.q[d];
             loop[r] = R.loop;
         }
         // per record, the directions q whose node B + c_q is active fluid: its tile is present
@@ -826,7 +868,6 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         v.q = upload(s, q, ok);
         v.loop = upload(s, loop, ok);
         v.nfluid = upload(s, nfluid, ok);
-        v.yc = upload(s, yc, ok);
         s->d_slip = (float *)dalloc(s, 2 * (size_t)std::max(n_loops, 1) * sizeof(float));
         v.slip = s->d_slip;
         float **outs[9] = {&v.drhoW, &v.uWx, &v.uWy, &v.utau, &v.chiB, &v.tx, &v.ty, &v.ut, &v.utau_start};
@@ -1071,9 +1112,8 @@ lbm_status lbm_step_launch(lbm_solver *s, int level, int kind)
         ls.wall = (l == L - 1) && s->rec.n > 0;
         ls.restrict_up = kind == 1 && C != nullptr;
         ls.pp = C ? s->parity[l - 1] : 0;
-        ls.shape = s->shape[l];
-        ls.status = s->d_status;
-        const lbmdev::LevelTune tu{s->min_blocks[l], 0, s->sched[l], s->shape[l]};
+            ls.status = s->d_status;
+        const lbmdev::LevelTune tu{block_warps(s->sched[l]), 0, plain_form(P.n_gen_warps + P.n_plain, s->k.sms)};
         lbmdev::launch_level(s->stream, P, F, C, s->rec, s->k, ls, tu);
         s->parity[l] ^= 1;
     }
@@ -1489,8 +1529,8 @@ lbm_status lbm_get_info(lbm_solver *s, lbm_info *out)
         out->cells_active[l] = act;
         out->cells_present[l] = pres;
         out->slots[l] = (long long)G.ntiles * LBM_TILE;
-        out->work_tiles[l] = s->lv[l].v.n_work_tiles;
-        out->work_warps[l] = s->lv[l].v.n_work_warps;
+        out->work_tiles[l] = (long long)s->lv[l].work_tiles.size();
+        out->work_warps[l] = (long long)s->lv[l].work_warps.size();
         nu += act << l;
     }
     out->node_updates_per_step = nu;
@@ -1721,6 +1761,10 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
     }
     lbmdev::BatchArgs a;
     a.n = 0;
+    int warps = 0;
+    for (lbm_solver *s : b->m)
+        if (l < s->L) warps += s->lv[l].v.n_gen_warps + s->lv[l].v.n_plain;
+    a.plain = plain_form(warps, b->m[0]->k.sms);
     unsigned grid = 0;
     for (lbm_solver *s : b->m) {
         if (l >= s->L) continue;
@@ -1737,13 +1781,12 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
         d.ls.wall = (l == L - 1) && s->rec.n > 0;
         d.ls.restrict_up = restrict_up && l > 0;
         d.ls.pp = l > 0 ? s->parity[l - 1] : 0;
-        d.ls.shape = 0;
         d.ls.status = s->d_status;
         d.ls.tl = nullptr;
         d.ls.tl_base = 0;
         d.kind = d.ls.wall ? 2 : (d.ls.has_child ? 1 : 0);
         d.first_block = (int)grid;
-        grid += (unsigned)std::max(d.P.n_work_tiles, 0);
+        grid += (unsigned)((d.P.n_gen_warps + (a.plain ? d.P.n_plain / 2 : d.P.n_plain) + LBM_BLOCK / 32 - 1) / (LBM_BLOCK / 32));
         s->parity[l] ^= 1;
     }
     if (grid) { lbmdev::launch_level_batch(st, a, b->store, grid, 1); nk++; }
@@ -2038,7 +2081,7 @@ lbm_status lbm_set_timeline(lbm_solver *s, int on)
         long long need = 0;
         for (int l = 0; l < s->L; l++) {
             const lbmdev::LevelView &v = s->lv[l].v;
-            need += (1LL << l) * (std::max(v.n_work_tiles, (v.n_work_warps + 1) / 2) + v.n_band_tiles);
+            need += (1LL << l) * ((v.n_gen_warps + v.n_plain + 1) / 2 + v.n_band_tiles);
         }
         need *= 2;
         s->d_tl = (unsigned long long *)dalloc(s, (size_t)need * 3 * sizeof(unsigned long long));
