@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -125,6 +126,7 @@ struct lbm_solver {
     bool off_schedule = false;    // single launches (lbm_step_launch) left the level schedule
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     std::vector<void *> allocs;
+    lbmgrid::cellvec<float> host_fields;   // fields of a level on their way to the caller (download_level)
     double device_bytes = 0;
     int *d_status = nullptr;
     double *d_acc = nullptr;
@@ -233,6 +235,7 @@ static void free_all(lbm_solver *s)
         else cudaFree(p);
     }
     s->allocs.clear();
+    lbmgrid::cellvec<float>().swap(s->host_fields);
     s->device_bytes = 0;
     s->geometry = false;
     s->d_tl = nullptr;
@@ -754,23 +757,20 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
 #pragma omp parallel for schedule(static)
             for (long m = 0; m < nw; m++) {
                 const int t = ww[m] >> 3, w = ww[m] & 7;
-                bool ok_w = true;
-                for (int c = 0; ok_w && c < 32; c++) {
-                    const int lx = (w & 1) * 16 + (c & 15), ly = (w >> 1) * 2 + (c >> 4);
-                    ok_w = H.flags[(size_t)t * LBM_TILE + ly * LBM_TX + lx] == KIND_ACTIVE;
-                    for (int d = 1; ok_w && d < 9; d++) {
-                        const int ax = lx + CXh[d], ay = ly + CYh[d];
-                        const int sx = ax < 0 ? -1 : (ax >= LBM_TX ? 1 : 0), sy = ay < 0 ? -1 : (ay >= LBM_TY ? 1 : 0);
-                        for (int e = 1; e < 9; e++)
-                            if (CXh[e] == sx && CYh[e] == sy && G.nbr[(size_t)t * 9 + e] < 0) ok_w = false;
+                bool ok_w = true, bn = false;
+                for (int r = 0; r < 2; r++) {
+                    const uint32_t *f = &H.flags[(size_t)t * LBM_TILE + ((w >> 1) * 2 + r) * LBM_TX + (w & 1) * 16];
+                    for (int c = 0; c < 16; c++) {
+                        ok_w = ok_w && f[c] == KIND_ACTIVE;
+                        bn = bn || (f[c] & (FL_KIND_MASK | FL_SOLID | FL_BNODE)) == (KIND_ACTIVE | FL_BNODE);
                     }
                 }
+                // the block's neighbours reach into the tiles beside, below or above it
+                const int sx = (w & 1) ? 1 : -1, sy = (w >> 1) == 0 ? -1 : ((w >> 1) == 3 ? 1 : 0);
+                for (int e = 1; e < 9; e++)
+                    if ((CXh[e] == 0 || CXh[e] == sx) && (CYh[e] == 0 || CYh[e] == sy) && G.nbr[(size_t)t * 9 + e] < 0) ok_w = false;
                 plain[m] = ok_w;
-                for (int c = 0; c < 32; c++) {
-                    const int lx = (w & 1) * 16 + (c & 15), ly = (w >> 1) * 2 + (c >> 4);
-                    const uint32_t f = H.flags[(size_t)t * LBM_TILE + ly * LBM_TX + lx];
-                    if ((f & (FL_KIND_MASK | FL_SOLID | FL_BNODE)) == (KIND_ACTIVE | FL_BNODE)) has_bnode[m] = 1;
-                }
+                has_bnode[m] = bn;
             }
             std::vector<int> gw, pw;
             for (long m = 0; m < nw; m++)
@@ -794,11 +794,10 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         v.f = dalloc(s, 9 * ns * pop_bytes(c.store));
         ok = ok && v.f;
         for (int b = 0; b < 2; b++) {
-            v.chi[b] = (float *)dalloc(s, ns * sizeof(float));
-            v.drho[b] = (float *)dalloc(s, ns * sizeof(float));
-            v.ux[b] = (float *)dalloc(s, ns * sizeof(float));
-            v.uy[b] = (float *)dalloc(s, ns * sizeof(float));
-            ok = ok && v.chi[b] && v.drho[b] && v.ux[b] && v.uy[b];
+            // the four fields of a time level in one piece: queries copy them at once
+            float *fields = (float *)dalloc(s, 4 * ns * sizeof(float));
+            ok = ok && fields;
+            v.drho[b] = fields; v.ux[b] = fields + ns; v.uy[b] = fields + 2 * ns; v.chi[b] = fields + 3 * ns;
         }
         v.n_band = n_band[l];
         v.ebuf = (float *)dalloc(s, 9 * (size_t)std::max(n_band[l], 1) * sizeof(float));
@@ -1162,18 +1161,21 @@ lbm_status lbm_get_level_box(lbm_solver *s, int level, int *i0, int *j0, int *nx
     return LBM_OK;
 }
 
-static lbm_status download_level(lbm_solver *s, int l, std::vector<float> &dr, std::vector<float> &ux,
-                                 std::vector<float> &uy, std::vector<float> &chi)
+// rho - 1, u_x, u_y, chi of a level at the current time into the handle's host buffer, one after
+// the other (v.ns values each).  The buffer is kept with the handle, sized for the largest level
+// asked for: copies into memory touched before run at 176 GB/s here, into fresh pages at 6 .. 18.
+static lbm_status download_level(lbm_solver *s, int l, float **out)
 {
     const LevelView &v = s->lv[l].v;
-    const int p = s->parity[l];
-    const size_t nb = (size_t)v.ns * sizeof(float);
-    dr.resize(v.ns); ux.resize(v.ns); uy.resize(v.ns); chi.resize(v.ns);
-    CK(cudaMemcpyAsync(dr.data(), v.drho[p], nb, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(ux.data(), v.ux[p], nb, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(uy.data(), v.uy[p], nb, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(chi.data(), v.chi[p], nb, cudaMemcpyDeviceToHost, s->stream));
+    const size_t n = 4 * (size_t)v.ns;
+    try {
+        if (s->host_fields.size() < n) s->host_fields.resize(n);
+    } catch (const std::bad_alloc &) {
+        return fail(s, LBM_ERR_OOM, "host memory for the fields");
+    }
+    CK(cudaMemcpyAsync(s->host_fields.data(), v.drho[s->parity[l]], n * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    *out = s->host_fields.data();
     return LBM_OK;
 }
 
@@ -1196,23 +1198,32 @@ lbm_status lbm_get_fields(lbm_solver *s, int level, double *rho, double *ux, dou
     if ((long long)nx * ny > cap) return fail(s, LBM_ERR_INVALID_ARG, "capacity too small");
     const bool fields = rho || ux || uy || chi;
     if (fields && !s->geometry) return fail(s, LBM_ERR_NO_GEOMETRY, "no device state (host-only handle): only the mask");
-    std::vector<float> dr, u, v, c2;
+    float *f = nullptr;
     if (fields) {
-        st = download_level(s, level, dr, u, v, c2);
+        st = download_level(s, level, &f);
         if (st != LBM_OK) return st;
     }
     const lbmgrid::Level &G = s->g.lv[level];
+    const size_t ns = (size_t)s->lv[level].v.ns;
+    // rows in parallel, a row in pieces of one tile (consecutive slots): converting and placing the
+    // values was the larger part of a read (2048^2 cells: 32 ms on one thread with a slot lookup a
+    // cell and fresh buffers, 3.2 ms this way on 16)
+#pragma omp parallel for schedule(static) if ((long long)nx * ny > 16384)
     for (int j = 0; j < ny; j++)
-        for (int i = 0; i < nx; i++) {
-            long sl = G.slot(i0 + i, j0 + j);
-            long long o = (long long)j * nx + i;
-            unsigned char m = mask_of(G, G.idx(i0 + i, j0 + j));
-            if (mask) mask[o] = m;
-            bool has = m >= 1 && m <= 4 && sl >= 0;
-            if (rho) rho[o] = has ? 1.0 + (double)dr[sl] : NAN;
-            if (ux) ux[o] = has ? (double)u[sl] : NAN;
-            if (uy) uy[o] = has ? (double)v[sl] : NAN;
-            if (chi) chi[o] = has ? (double)c2[sl] : NAN;
+        for (int i = 0, n = 0; i < nx; i += n) {
+            n = std::min(nx - i, LBM_TX - ((i0 + i) & (LBM_TX - 1)));
+            const long sl = G.slot(i0 + i, j0 + j);
+            const long long o = (long long)j * nx + i;
+            for (int c = 0; c < n; c++) {
+                const unsigned char m = mask_of(G, G.idx(i0 + i + c, j0 + j));
+                const bool has = m >= 1 && m <= 4 && sl >= 0;
+                const size_t q = (size_t)sl + c;
+                if (mask) mask[o + c] = m;
+                if (rho) rho[o + c] = has ? 1.0 + (double)f[q] : NAN;
+                if (ux) ux[o + c] = has ? (double)f[ns + q] : NAN;
+                if (uy) uy[o + c] = has ? (double)f[2 * ns + q] : NAN;
+                if (chi) chi[o + c] = has ? (double)f[3 * ns + q] : NAN;
+            }
         }
     return LBM_OK;
 }
@@ -1325,13 +1336,16 @@ lbm_status lbm_set_fields(lbm_solver *s, int level, const double *rho, const dou
     if (st != LBM_OK) return st;
     const LevelView &v = s->lv[level].v;
     const int p = s->parity[level];
-    std::vector<float> dr, u, w, c2, c3(v.ns), post;
-    st = download_level(s, level, dr, u, w, c2);
+    std::vector<float> c3(v.ns), post;
+    float *f = nullptr;
+    st = download_level(s, level, &f);
     if (st != LBM_OK) return st;
+    float *dr = f, *u = f + v.ns, *w = f + 2 * (size_t)v.ns, *c2 = f + 3 * (size_t)v.ns;
     CK(cudaMemcpyAsync(c3.data(), v.chi[p ^ 1], v.ns * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
     if ((st = gather_post(s, level, post)) != LBM_OK) return st;
     const lbmgrid::Level &G = s->g.lv[level];
     const std::vector<uint32_t> &fl = s->lv[level].flags;
+#pragma omp parallel for schedule(static) if ((long long)nx * ny > 16384)
     for (int j = 0; j < ny; j++)
         for (int i = 0; i < nx; i++) {
             long sl = G.slot(i0 + i, j0 + j);
@@ -1348,10 +1362,7 @@ lbm_status lbm_set_fields(lbm_solver *s, int level, const double *rho, const dou
             feq_shifted(r, a, b, g9);
             for (int q = 0; q < 9; q++) post[(size_t)q * v.ns + sl] = g9[q];
         }
-    CK(cudaMemcpyAsync(v.drho[p], dr.data(), v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
-    CK(cudaMemcpyAsync(v.ux[p], u.data(), v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
-    CK(cudaMemcpyAsync(v.uy[p], w.data(), v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
-    CK(cudaMemcpyAsync(v.chi[p], c2.data(), v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
+    CK(cudaMemcpyAsync(v.drho[p], f, 4 * (size_t)v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
     CK(cudaMemcpyAsync(v.chi[p ^ 1], c3.data(), v.ns * sizeof(float), cudaMemcpyHostToDevice, s->stream));
     size_t ns_max = 0;
     for (int l = 0; l < s->L; l++) ns_max = std::max(ns_max, (size_t)s->lv[l].v.ns);
