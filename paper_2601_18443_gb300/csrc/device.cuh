@@ -19,8 +19,8 @@ struct LevelView {
     const int *nbr;               // 9 per tile, D2Q9 order, -1 absent
     const int *child;             // 4 per tile: tiles of level l+1, index b * 2 + a
     const int *parent;            // tile of level l-1 holding the parents, or -1
-    const int *band_tiles;        // tiles with band cells
-    int n_band_tiles;
+    const int *band_slot;         // per band cell: its slot if it is active fluid, else -1
+    const int4 *band_tgt;         // per band cell four rows of child-level slots (BandTargets)
     const int *work;              // tile * 8 + w of the 16 x 2-cell warps w that hold an active or ghost
     int n_gen_warps, n_pair_warps;// fluid cell: n_gen_warps entries in cost order, of which the first
                                   // n_pair_warps / 2 blocks (with boundary nodes) stand twice, then
@@ -109,6 +109,7 @@ void launch_level(cudaStream_t st, const LevelView &P, const LevelView *F, const
                   const StepConsts &k, const LevelStep &ls, const LevelTune &tu);
 void launch_prolong(cudaStream_t st, const LevelView &P, const LevelView &F, int p, int pdl,
                     unsigned long long *tl = nullptr, int tl_base = 0);
+unsigned prolong_blocks(const LevelView &P);    // blocks of a prolongation launch
 void launch_wallfn(cudaStream_t st, const LevelView &P, int p, const RecView &R, const StepConsts &k);
 void launch_restrict(cudaStream_t st, const LevelView &P, const LevelView &F, int pp, int pf);
 void launch_init_feq(cudaStream_t st, const LevelView &P, const float *feq9, float U, float chi_inf);

@@ -17,66 +17,93 @@ extern template void launch_level_batch_store<__nv_bfloat16>(cudaStream_t, const
 
 // ------------------------------------------------------------------ prolongation (Sec 2.2)
 // ghost children of the band cells of level l: linear LSQ reconstruction of chi and u
-// about the parent (fields at time t), rho copied; written to both time levels of l+1
-__device__ __forceinline__ void prolong_tile(const LevelView &P, const LevelView &F, int p, int t, int *nb3)
+// about the parent (fields at time t), rho copied; written to both time levels of l+1.
+// One thread a band cell, over the level's list of them: all addresses are static and found
+// before the wait for the preceding kernel, so that a launch is one round of loads, the
+// arithmetic and the stores (c/256 airfoil, level 4: 1.1 us; 1.8 us with one thread a cell of every
+// tile with a band cell, flags and child table read after the wait).  One warp a block spreads the
+// scattered accesses over more SMs (blocks of 128: 1.5 us).
+#define PROLONG_THREADS 32
+
+struct ProlongCell {
+    int s[9];           // own slot and those at offsets +c_q, or s[0] < 0: nothing to do
+    int row[2];         // slots of the first child of either row, or -1
+};
+
+__device__ __forceinline__ ProlongCell prolong_cell(const LevelView &P, int b)
 {
-    const int c = threadIdx.x;
-    const int lx = c & 31, ly = c >> 5;
-    const int slot = t * LBM_TILE + c;
-    const uint32_t fl = P.flags[slot];
-    if ((fl & FL_KIND_MASK) != KIND_ACTIVE || (fl & FL_SOLID) || !(fl & FL_BAND)) return;
-    const int cb = child_base(P, t, lx, ly);
-    if (cb < 0) return;
+    ProlongCell c;
+    c.s[0] = b < P.n_band ? __ldg(P.band_slot + b) : -1;
+    c.row[0] = c.row[1] = -1;
+    if (c.s[0] < 0) return c;
+    c.row[0] = __ldg(P.band_tgt + 4 * b + 1).y;
+    c.row[1] = __ldg(P.band_tgt + 4 * b + 2).y;
+    const int t = c.s[0] / LBM_TILE, lx = c.s[0] & (LBM_TX - 1), ly = (c.s[0] / LBM_TX) & (LBM_TY - 1);
+#pragma unroll
+    for (int q = 1; q < 9; q++) {
+        const int nx = lx + cxq(q), ny = ly + cyq(q);
+        const int sx = nx < 0 ? 0 : (nx >= LBM_TX ? 2 : 1), sy = ny < 0 ? 0 : (ny >= LBM_TY ? 2 : 1);
+        const int tt = sx == 1 && sy == 1 ? t : __ldg(P.nbr + t * 9 + dir_of3(sy * 3 + sx));
+        c.s[q] = tt < 0 ? c.s[0] : tt * LBM_TILE + (ny & (LBM_TY - 1)) * LBM_TX + (nx & (LBM_TX - 1));
+    }
+    return c;
+}
+
+__device__ __forceinline__ void prolong_write(const LevelView &P, const LevelView &F, int p, const ProlongCell &c)
+{
+    if (c.s[0] < 0) return;
     Stencil S;
-    gather(nb3, P.chi[p], P.ux[p], P.uy[p], lx, ly, slot, S);
+#pragma unroll
+    for (int q = 0; q < 9; q++) {
+        S.chi[q] = __ldg(P.chi[p] + c.s[q]); S.ux[q] = __ldg(P.ux[p] + c.s[q]); S.uy[q] = __ldg(P.uy[p] + c.s[q]);
+    }
+    const float dr = __ldg(P.drho[p] + c.s[0]);
     float gcx, gcy, gux, guy, gvx, gvy;
     lsq_grad(S.chi, gcx, gcy); lsq_grad(S.ux, gux, guy); lsq_grad(S.uy, gvx, gvy);
-    const float dr = P.drho[p][slot];
 #pragma unroll
-    for (int m = 0; m < 4; m++) {
-        const int a = m & 1, b = m >> 1;
-        const float ox = 0.5f * (a - 0.5f), oy = 0.5f * (b - 0.5f);
-        const int cs = cb + b * LBM_TX + a;
-        const float vc = S.chi[0] + gcx * ox + gcy * oy;
-        const float vu = S.ux[0] + gux * ox + guy * oy;
-        const float vv = S.uy[0] + gvx * ox + gvy * oy;
+    for (int b = 0; b < 2; b++) {
+        const int cs = c.row[b];
+        if (cs < 0) continue;
+        float vc[2], vu[2], vv[2];
+#pragma unroll
+        for (int a = 0; a < 2; a++) {
+            const float ox = 0.5f * (a - 0.5f), oy = 0.5f * (b - 0.5f);
+            vc[a] = S.chi[0] + gcx * ox + gcy * oy;
+            vu[a] = S.ux[0] + gux * ox + guy * oy;
+            vv[a] = S.uy[0] + gvx * ox + gvy * oy;
+        }
+        const float vr[2] = {dr, dr};
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            F.chi[h][cs] = vc; F.ux[h][cs] = vu; F.uy[h][cs] = vv; F.drho[h][cs] = dr;
+            st2(F.chi[h] + cs, vc); st2(F.ux[h] + cs, vu); st2(F.uy[h] + cs, vv); st2(F.drho[h] + cs, vr);
         }
     }
 }
 
-__global__ void __launch_bounds__(256) k_prolong(LevelView P, LevelView F, int p, unsigned long long *tl, int tl_base)
+__global__ void __launch_bounds__(PROLONG_THREADS) k_prolong(LevelView P, LevelView F, int p, unsigned long long *tl, int tl_base)
 {
     tl_mark(tl, tl_base, 0);
-    __shared__ int nb3[9];
-    const int t = P.band_tiles[blockIdx.x];
-    load_nb3(P, t, nb3);
-    __syncthreads();
+    const ProlongCell c = prolong_cell(P, blockIdx.x * PROLONG_THREADS + threadIdx.x);
     griddep_launch();
     griddep_wait();
     tl_mark(tl, tl_base, 1);
-    prolong_tile(P, F, p, t, nb3);
+    prolong_write(P, F, p, c);
     tl_end(tl, tl_base);
 }
 
-// batched form of k_prolong (same solve lookup as k_level_batch, over band tiles)
-__global__ void __launch_bounds__(256) k_prolong_batch(const __grid_constant__ ProlongBatchArgs a)
+// batched form of k_prolong (same solve lookup as k_level_batch)
+__global__ void __launch_bounds__(PROLONG_THREADS) k_prolong_batch(const __grid_constant__ ProlongBatchArgs a)
 {
     int i = 0;
     for (int m = 1; m < a.n; m++)
         if (a.d[m].first_block <= (int)blockIdx.x) i = m;
     const ProlongDesc &d = a.d[i];
     tl_mark(a.tl, a.tl_base, 0);
-    __shared__ int nb3[9];
-    const int t = d.P.band_tiles[blockIdx.x - d.first_block];
-    load_nb3(d.P, t, nb3);
-    __syncthreads();
+    const ProlongCell c = prolong_cell(d.P, ((int)blockIdx.x - d.first_block) * PROLONG_THREADS + threadIdx.x);
     griddep_launch();
     griddep_wait();
     tl_mark(a.tl, a.tl_base, 1);
-    prolong_tile(d.P, d.F, d.p, t, nb3);
+    prolong_write(d.P, d.F, d.p, c);
     tl_end(a.tl, a.tl_base);
 }
 
@@ -217,7 +244,8 @@ __global__ void k_explode(LevelView P, LevelView F, StepConsts k, const float *p
     if ((fl & FL_KIND_MASK) != KIND_ACTIVE || (fl & FL_SOLID) || !(fl & FL_BAND)) return;
     float o[9];
     for (int q = 0; q < 9; q++) o[q] = post[(size_t)q * P.ns + slot];
-    explode_band<T>(P, F, k, t, lx, ly, fl, __ldg(P.aux + slot), o);
+    const int b = __ldg(P.aux + slot);
+    explode_band<T>(P, F, k, fl, b, band_targets(P, b), o);
 }
 
 // rest state: every present cell's populations are e (values to store, relative to the
@@ -362,13 +390,16 @@ void launch_level_batch(cudaStream_t st, const BatchArgs &a, int store, unsigned
 
 void launch_prolong_batch(cudaStream_t st, const ProlongBatchArgs &a, unsigned grid, int pdl)
 {
-    if (grid > 0) launch_pdl(k_prolong_batch, grid, st, pdl, a);
+    if (grid > 0) launch_pdl_bs(k_prolong_batch, grid, PROLONG_THREADS, st, pdl, a);
 }
+
+unsigned prolong_blocks(const LevelView &P) { return (unsigned)((P.n_band + PROLONG_THREADS - 1) / PROLONG_THREADS); }
 
 void launch_prolong(cudaStream_t st, const LevelView &P, const LevelView &F, int p, int pdl, unsigned long long *tl,
                     int tl_base)
 {
-    if (P.n_band_tiles > 0) launch_pdl(k_prolong, (unsigned)P.n_band_tiles, st, pdl, P, F, p, tl, tl_base);
+    const unsigned grid = prolong_blocks(P);
+    if (grid > 0) launch_pdl_bs(k_prolong, grid, PROLONG_THREADS, st, pdl, P, F, p, tl, tl_base);
 }
 
 void launch_wallfn(cudaStream_t st, const LevelView &P, int p, const RecView &R, const StepConsts &k)

@@ -319,7 +319,7 @@ static void flush_prolong(lbm_solver *s, cudaStream_t st, long long &nk)
         s->pend.tl_base = base;
         lbmdev::launch_prolong_batch(st, s->pend, s->pend_grid, s->pdl);
     }
-    mark_end(s, KC_PROLONG, (long long)s->pend_grid * LBM_TILE, s->pend_level);
+    mark_end(s, KC_PROLONG, (long long)s->pend_grid * 32, s->pend_level);
     nk++;
     s->pend.n = 0;
     s->pend_grid = 0;
@@ -352,13 +352,13 @@ static void advance(lbm_solver *s, cudaStream_t st, int l, int restrict_up, long
         // the prolongation joins the pending ones when it reads nothing they write (it
         // follows the prolongation of level l - 1 in the descent); the next level step
         // launches them
-        if (P.n_band_tiles > 0) {
+        if (P.n_band > 0) {
             if (s->pend.n > 0 && !(s->prolong_merge && s->prolong_indep[l] && s->pend_level + s->pend.n == l))
                 flush_prolong(s, st, nk);
             if (s->pend.n == 0) s->pend_level = l;
             lbmdev::ProlongDesc &d = s->pend.d[s->pend.n++];
             d.P = P; d.F = *F; d.p = s->parity[l]; d.first_block = (int)s->pend_grid;
-            s->pend_grid += (unsigned)P.n_band_tiles;
+            s->pend_grid += lbmdev::prolong_blocks(P);
         }
         advance(s, st, l + 1, 0, nk);
         advance(s, st, l + 1, 1, nk);
@@ -741,8 +741,26 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         v.nbr = upload(s, G.nbr, ok);
         v.child = upload(s, G.child, ok);
         v.parent = upload(s, G.parent, ok);
-        v.band_tiles = upload(s, G.band_tiles, ok);
-        v.n_band_tiles = (int)G.band_tiles.size();
+        {
+            // band cells: slots, and those of the child-level cells that the explosion and the
+            // prolongation write (rows cy0 - 1 .. cy0 + 2; columns cx0 - 1, cx0, cx0 + 2)
+            const std::vector<int> &bij = H.band_ij;
+            std::vector<int> bs(n_band[l], -1);
+            std::vector<int4> bt(4 * (size_t)n_band[l], int4{-1, -1, -1, -1});
+#pragma omp parallel for schedule(static)
+            for (int b = 0; b < n_band[l]; b++) {
+                const int i = bij[2 * (size_t)b], j = bij[2 * (size_t)b + 1];
+                const long sl = G.slot(i, j);
+                if (sl < 0 || !Gf || Gf->slot(2LL * i, 2LL * j) < 0) continue;
+                if ((H.flags[sl] & (FL_KIND_MASK | FL_SOLID)) == KIND_ACTIVE) bs[b] = (int)sl;
+                for (int a = 0; a < 4; a++) {
+                    const long long y = 2LL * j + a - 1;
+                    bt[4 * (size_t)b + a] = int4{(int)Gf->slot(2LL * i - 1, y), (int)Gf->slot(2LL * i, y), (int)Gf->slot(2LL * i + 2, y), -1};
+                }
+            }
+            v.band_slot = upload(s, bs, ok);
+            v.band_tgt = upload(s, bt, ok);
+        }
         {
             // work tiles in the same cost order as the warps below (a block's warps start
             // together, so the expensive tiles go first and the last blocks are cheap)
@@ -1809,10 +1827,10 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
         a.tl_base = 0;
         unsigned grid = 0;
         for (lbm_solver *s : b->m) {
-            if (l + 1 >= s->L || s->lv[l].v.n_band_tiles <= 0) continue;
+            if (l + 1 >= s->L || s->lv[l].v.n_band <= 0) continue;
             lbmdev::ProlongDesc &d = a.d[a.n++];
             d.P = s->lv[l].v; d.F = s->lv[l + 1].v; d.p = s->parity[l]; d.first_block = (int)grid;
-            grid += (unsigned)s->lv[l].v.n_band_tiles;
+            grid += lbmdev::prolong_blocks(s->lv[l].v);
         }
         if (grid) { lbmdev::launch_prolong_batch(st, a, grid, 1); nk++; }
     }
@@ -2142,7 +2160,7 @@ lbm_status lbm_set_timeline(lbm_solver *s, int on)
         long long need = 0;
         for (int l = 0; l < s->L; l++) {
             const lbmdev::LevelView &v = s->lv[l].v;
-            need += (1LL << l) * ((v.n_gen_warps + v.n_plain + 1) / 2 + v.n_band_tiles);
+            need += (1LL << l) * ((v.n_gen_warps + v.n_plain + 1) / 2 + lbmdev::prolong_blocks(v));
         }
         need *= 2;
         s->d_tl = (unsigned long long *)dalloc(s, (size_t)need * 3 * sizeof(unsigned long long));

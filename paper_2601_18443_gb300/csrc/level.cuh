@@ -290,17 +290,6 @@ struct Stencil {
     float chi[9], ux[9], uy[9];
 };
 
-__device__ __forceinline__ void gather(const int *nb3, const float *chi, const float *ux, const float *uy, int lx,
-                                       int ly, int slot, Stencil &S)
-{
-#pragma unroll
-    for (int q = 0; q < 9; q++) {
-        int s = q == 0 ? slot : nb_slot(nb3, lx, ly, cxq(q), cyq(q));
-        if (s < 0) s = slot;
-        S.chi[q] = __ldg(chi + s); S.ux[q] = __ldg(ux + s); S.uy[q] = __ldg(uy + s);
-    }
-}
-
 // level-0 box edge: neighbours across the top/bottom symmetry planes are mirror images
 __device__ __forceinline__ void gather0(const float *chi, const float *ux, const float *uy, const StepConsts &k, int i,
                                         int j, Stencil &S)
@@ -615,14 +604,26 @@ __device__ __forceinline__ void put_obuf(const StepConsts &k, int par, uint32_t 
 // reads them (slot (g + c_q, q) for child g).  Children that are solid or have no tile relay
 // nothing, so their share of the next coalescence is this value too.
 //
-// The targets of all four children lie in the 4 x 4 cells around them: their tiles are looked
-// up once for the 3 x 3 (tile column, tile row) combinations, so that the stores depend on one
-// round of loads, and the two children of a row share one 64-bit store where c_x = 0.
-template <typename T>
-__device__ __forceinline__ void explode_band(const LevelView &P, const LevelView &F, const StepConsts &k, int t, int lx,
-                                             int ly, uint32_t fl, int b, const float o[9], int *ls_status = nullptr)
+// The targets of all four children lie in the 4 x 4 cells around them.  Their slots are static:
+// tgt holds, per row cy0 - 1 .. cy0 + 2 of the cells (cx0 .. cx0 + 1, cy0 .. cy0 + 1), the slots
+// of cx0 - 1, of cx0 (and cx0 + 1, the next one) and of cx0 + 2, -1 where there is no tile, so that
+// the stores wait for no table; the two children of a row share one 64-bit store where c_x = 0.
+struct BandTargets {
+    int4 row[4];
+};
+
+__device__ __forceinline__ BandTargets band_targets(const LevelView &P, int b)
 {
-    b = checked_index(b, P.n_band, ls_status);
+    BandTargets t;
+#pragma unroll
+    for (int a = 0; a < 4; a++) t.row[a] = __ldg(P.band_tgt + 4 * b + a);
+    return t;
+}
+
+template <typename T>
+__device__ __forceinline__ void explode_band(const LevelView &P, const LevelView &F, const StepConsts &k, uint32_t fl, int b,
+                                             const BandTargets &tgt, const float o[9], int *status = nullptr)
+{
     float *eb = P.ebuf + b * 9;
 #pragma unroll
     for (int q = 0; q < 9; q++) eb[q] = o[q];
@@ -635,37 +636,18 @@ __device__ __forceinline__ void explode_band(const LevelView &P, const LevelView
             for (int q = 0; q < 9; q++) gb[q] = o[q];
         }
     }
-    int ct = P.child[t * 4 + ((2 * ly) >> 3) * 2 + ((2 * lx) >> 5)];
-    if (ct < 0) return;
-    ct = checked_index(ct, F.ntiles, ls_status);
     const Lat<T> LF{static_cast<T *>(F.f), F.ns, k.pshift};
-    const int cx0 = (2 * lx) & (LBM_TX - 1), cy0 = (2 * ly) & (LBM_TY - 1);
-    // first slot of the row at offset a (-1 .. 2) from cy0 in the tile column at offset c
-    // (0 the cells cx0, cx0 + 1; -1 the cell cx0 - 1; 1 the cell cx0 + 2), or -1
-    int base[3][4];
-#pragma unroll
-    for (int c = -1; c <= 1; c++) {
-        const int ax = c < 0 ? cx0 - 1 : (c > 0 ? cx0 + 2 : cx0);
-        const int sx = ax < 0 ? 0 : (ax >= LBM_TX ? 2 : 1);
-#pragma unroll
-        for (int a = -1; a <= 2; a++) {
-            const int ay = cy0 + a;
-            const int sy = ay < 0 ? 0 : (ay >= LBM_TY ? 2 : 1);
-            int tt = (sx == 1 && sy == 1) ? ct : __ldg(F.nbr + ct * 9 + dir_of3(sy * 3 + sx));
-            if (tt >= 0) tt = checked_index(tt, F.ntiles, ls_status);
-            base[c + 1][a + 1] = tt < 0 ? -1 : tt * LBM_TILE + (ay & (LBM_TY - 1)) * LBM_TX + (ax & (LBM_TX - 1));
-        }
-    }
 #pragma unroll
     for (int q = 0; q < 9; q++) {
 #pragma unroll
         for (int my = 0; my < 2; my++) {
-            const int a = my + cyq(q) + 1;
+            const int4 t = tgt.row[my + cyq(q) + 1];
+            const int in = t.y < 0 ? -1 : checked_index(t.y, F.ns - 1, status);
             if (cxq(q) == 0) {
-                if (base[1][a] >= 0) LF.st2(q, base[1][a], q, o[q], o[q]);
+                if (in >= 0) LF.st2(q, in, q, o[q], o[q]);
             } else {
                 // the children at cx0 and cx0 + 1 write to cx0 + c_x and cx0 + 1 + c_x
-                const int in = base[1][a], out = cxq(q) > 0 ? base[2][a] : base[0][a];
+                const int far = cxq(q) > 0 ? t.z : t.x, out = far < 0 ? -1 : checked_index(far, F.ns, status);
                 if (in >= 0) LF.st(q, cxq(q) > 0 ? in + 1 : in, q, o[q]);
                 if (out >= 0) LF.st(q, out, q, o[q]);
             }
@@ -678,6 +660,76 @@ __device__ __forceinline__ void explode_band(const LevelView &P, const LevelView
 __device__ __forceinline__ bool uses_aux(uint32_t fl)
 {
     return (fl & FL_KIND_MASK) == KIND_GHOST || (fl & (FL_BNODE | FL_BAND | (0xFFu << FL_COAL_SHIFT)));
+}
+
+// ------------------------------------------------------------------ work of a warp
+// The static part of a warp's work, read before the wait for the preceding kernel.  The work list
+// holds the general 16 x 2-cell blocks (each with boundary nodes twice: its wall warp, then its
+// partner), then the plain ones.  A PLAIN launch takes the latter two to a warp (plain_warp),
+// any other one to a warp as it takes the general ones.
+struct GeneralWork {
+    int t;              // tile
+    bool wall;          // one of a pair of warps
+    int lx, ly;         // the lane's cell
+    uint32_t fl;
+    int ax;
+    int s[9];           // own slot and those at offsets +c_q (the own one where there is no tile)
+    unsigned present;   // mask of the neighbours that have a tile
+    int ps;             // with a restriction: slot of the cell's parent, or -1
+};
+
+struct PlainWork {
+    int e;              // tile * 8 + block of the tile
+    int tv, th0, thv;   // tiles across the lane's vertical / horizontal / both tile edges, its own
+                        // where it has none
+};
+
+// warps that a launch over a level takes
+__host__ __device__ __forceinline__ int level_warps(const LevelView &P, bool plain)
+{
+    return P.n_gen_warps + (plain ? P.n_plain / 2 : P.n_plain);
+}
+
+__device__ __forceinline__ GeneralWork general_work(const LevelView &P, const LevelView &C, const LevelStep &ls, int w, int lane,
+                                                    int *nb3)
+{
+    GeneralWork W;
+    const int e = checked_index(__ldg(P.work + w), 8 * P.ntiles, ls.status), t = e >> 3;
+    W.t = t;
+    W.wall = w < P.n_pair_warps;
+    cell_of_thread((e & 7) * 32 + lane, W.lx, W.ly);
+    if (lane < 9) nb3[lane] = P.nbr[t * 9 + dir_of3(lane)];
+    const int slot = t * LBM_TILE + W.ly * LBM_TX + W.lx;
+    W.fl = __ldg(P.flags + slot);
+    W.ax = uses_aux(W.fl) ? __ldg(P.aux + slot) : -1;
+    __syncwarp();
+    W.present = neighbours(nb3, W.lx, W.ly, slot, W.s);
+#ifdef LBM_BOUNDS_CHECK
+#pragma unroll
+    for (int q = 1; q < 9; q++) W.s[q] = checked_index(W.s[q], P.ns, ls.status);
+#endif
+    W.ps = -1;
+    if (ls.restrict_up) {
+        const int pt = __ldg(P.parent + t);
+        const int px = (__ldg(P.tile_x + t) & 1) * (LBM_TX / 2) + (W.lx >> 1);
+        const int py = (__ldg(P.tile_y + t) & 1) * (LBM_TY / 2) + (W.ly >> 1);
+        if (pt >= 0) W.ps = checked_index(pt, C.ntiles, ls.status) * LBM_TILE + py * LBM_TX + px;
+    }
+    return W;
+}
+
+__device__ __forceinline__ PlainWork plain_work(const LevelView &P, const LevelStep &ls, int w, int lane)
+{
+    PlainWork W;
+    W.e = checked_index(__ldg(P.work + P.n_gen_warps + 2 * (w - P.n_gen_warps) + (lane >> 4)), 8 * P.ntiles, ls.status);
+    const int t = W.e >> 3, li = lane & 15;
+    const int lx = (W.e & 1) * 16 + (li & 7) * 2, ly = ((W.e >> 1) & 3) * 2 + (li >> 3);
+    const int sx = lx == 0 ? 0 : (lx == LBM_TX - 2 ? 2 : 1), sy = ly == 0 ? 0 : (ly == LBM_TY - 1 ? 2 : 1);
+    const int *nb = P.nbr + t * 9;
+    W.tv = sy == 1 ? t : __ldg(nb + dir_of3(sy * 3 + 1));
+    W.th0 = sx == 1 ? t : __ldg(nb + dir_of3(3 + sx));
+    W.thv = sx == 1 ? W.tv : (sy == 1 ? W.th0 : __ldg(nb + dir_of3(sy * 3 + sx)));
+    return W;
 }
 
 // ------------------------------------------------------------------ wall warps
@@ -771,8 +823,7 @@ __device__ __forceinline__ void wall_warp(const LevelView &P, const RecView &R, 
 
 // One 16 x 2-cell warp of the fused level step, one cell a lane, for blocks of cells with
 // anything besides plain active cells in them: every kind of cell, level-0 edges, walls,
-// interfaces.  nb3 holds the 3 x 3 neighbour tiles of t for this warp, fl and ax the cell's
-// flag and aux words.
+// interfaces.
 //
 // A launch of a small level is one such warp's latency (a round trip to L2 is about 0.5 us, and a
 // warp alone issues an instruction every three to four cycles), so the loads come first and in as
@@ -782,15 +833,19 @@ __device__ __forceinline__ void wall_warp(const LevelView &P, const RecView &R, 
 // go out together, for every lane and whatever its kind; the coalescence buffers follow as one
 // round instead of one per direction, and the wall function runs in a warp of its own (wall_warp).
 // c/256 airfoil: the finest level's launch 9.7 / 12.9 us (even / odd) with the code of one cell a
-// thread and the boundary nodes' work in line, 3.0 / 3.5 us this way.
+// thread and the boundary nodes' work in line, 2.8 / 3.2 us this way; level 4 (interfaces on both
+// sides) 4.9 / 6.6 us, then 3.3 / 4.6 with neighbour slots, parents and the explosion's targets
+// found after the wait, now 2.6 / 3.3 us.
 template <int KIND, typename T, bool ODD, bool EDGE>
 __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView &F, const LevelView &C, const RecView &R,
-                                             const StepConsts &k, const LevelStep &ls, const Lat<T> &L, int t, int lane,
-                                             int lx, int ly, const int *nb3, uint32_t fl, int ax, const WallPair *wp,
-                                             int pair, const CutLinks &cut)
+                                             const StepConsts &k, const LevelStep &ls, const Lat<T> &L, const GeneralWork &W,
+                                             int lane, const WallPair *wp, int pair, const CutLinks &cut)
 {
     constexpr bool CHILD = KIND == 1, WALL = KIND == 2;
-    const int slot = t * LBM_TILE + ly * LBM_TX + lx;
+    const int *nbs = W.s, slot = W.s[0], t = W.t, lx = W.lx, ly = W.ly;
+    const unsigned present = W.present;
+    const uint32_t fl = W.fl;
+    int ax = W.ax;
     const uint32_t kind = fl & FL_KIND_MASK;
     const bool fluid = !(fl & FL_SOLID);
     const bool act = kind == KIND_ACTIVE && fluid, ghost = kind == KIND_GHOST && fluid;
@@ -799,12 +854,6 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
 
     const bool edge = EDGE && act && (fl & (FL_INLET | FL_OUTLET | FL_BOTTOM | FL_TOP));
     const bool bnode = WALL && act && (fl & FL_BNODE);
-    int nbs[9];
-    const unsigned present = neighbours(nb3, lx, ly, slot, nbs);
-#ifdef LBM_BOUNDS_CHECK
-#pragma unroll
-    for (int q = 1; q < 9; q++) nbs[q] = checked_index(nbs[q], P.ns, ls.status);
-#endif
     // ---- streaming (eq 1): the populations arriving at the cell.  (Where no upstream tile
     // exists the own slot is read and the value replaced below.)
     float g[9];
@@ -857,17 +906,20 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
             }
         }
     }
+    const bool band = CHILD && act && (fl & FL_BAND);
+    if (CHILD && act && (fl & (FL_BAND | (0xFFu << FL_COAL_SHIFT)))) ax = checked_index(ax, P.n_band, ls.status);
     if (CHILD && (fl & (0xFFu << FL_COAL_SHIFT)) && act) {
         // coalescence: mean of what the four ghost children pulled in the fine level's odd sub-step
-        const float *gb = P.gbuf + checked_index(ax, P.n_band, ls.status) * 36;
-        float c[9][4];
+        const float4 *gb = reinterpret_cast<const float4 *>(P.gbuf + ax * 36);
+        float c[36];                                      // child m's population q at 9 m + q
+#pragma unroll
+        for (int i = 0; i < 9; i++) {
+            const float4 v = gb[i];
+            c[4 * i] = v.x; c[4 * i + 1] = v.y; c[4 * i + 2] = v.z; c[4 * i + 3] = v.w;
+        }
 #pragma unroll
         for (int q = 1; q < 9; q++)
-#pragma unroll
-            for (int m = 0; m < 4; m++) c[q][m] = gb[9 * m + q];
-#pragma unroll
-        for (int q = 1; q < 9; q++)
-            if (fl & (1u << (FL_COAL_SHIFT + q - 1))) g[q] = 0.25f * (c[q][0] + c[q][1] + c[q][2] + c[q][3]);
+            if (fl & (1u << (FL_COAL_SHIFT + q - 1))) g[q] = 0.25f * (c[q] + c[9 + q] + c[18 + q] + c[27 + q]);
     }
     // ---- SA-neg update of chi (Sec 2.2), fields at time t
     float chin = 0.0f;
@@ -876,6 +928,8 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
         else if (edge && (fl & FL_INLET)) chin = k.chi_inf;
         else chin = sa_update(S, id2, P.nu, k.sa_convection);
     }
+    BandTargets tgt = {};
+    if (band) tgt = band_targets(P, ax);
     // ---- wall function of the boundary nodes (Sec 2.3), fields at time t, from the partner warp
     // (all lanes wait, whatever their cells)
     float drW = 0.f, uWx = 0.f, uWy = 0.f;
@@ -967,7 +1021,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
         }
         if (EDGE && (fl & (FL_OUTLET | FL_OUTLET2)))
             put_obuf(k, p ^ 1, fl, P.tile_y[t] * LBM_TY + ly, o);
-        if (CHILD && (fl & FL_BAND)) explode_band<T>(P, F, k, t, lx, ly, fl, ax, o, ls.status);
+        if (band) explode_band<T>(P, F, k, fl, ax, tgt, o, ls.status);
         n_dr = drho; n_ux = ux; n_uy = uy; n_chi = chin;
     }
 
@@ -986,17 +1040,8 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
             a4 += __shfl_down_sync(0xffffffffu, a4, d); a5 += __shfl_down_sync(0xffffffffu, a5, d);
         }
         if (!(lane & 1) && lane < 16 && kind == KIND_ACTIVE) {
-#ifdef LBM_BOUNDS_CHECK
-            const int pt = P.parent[t] < 0 ? -1 : checked_index(P.parent[t], C.ntiles, ls.status);
-#else
-            const int pt = P.parent[t];
-#endif
-            const int n = (int)a5;
-            if (pt >= 0 && n > 0) {
-                const int px = (P.tile_x[t] & 1) * (LBM_TX / 2) + (lx >> 1);
-                const int py = (P.tile_y[t] & 1) * (LBM_TY / 2) + (ly >> 1);
-                const int ps = pt * LBM_TILE + py * LBM_TX + px;
-                const int q1 = ls.pp ^ 1;
+            const int n = (int)a5, ps = W.ps, q1 = ls.pp ^ 1;
+            if (ps >= 0 && n > 0) {
                 C.drho[q1][ps] = a0 / n; C.ux[q1][ps] = a2 / a1; C.uy[q1][ps] = a3 / a1;
                 C.chi[q1][ps] = a4 / n;
             }
@@ -1033,14 +1078,14 @@ __device__ __forceinline__ void row4(const float *a, int left, int mid, int righ
 // two cells a lane at 96 registers took 114, 165 and 82 us.
 template <typename T, bool ODD>
 __device__ __forceinline__ void plain_warp(const LevelView &P, const LevelView &C, const StepConsts &k, const LevelStep &ls,
-                                           const Lat<T> &L, int e, int lane, int tv, int th0, int thv, T *buf)
+                                           const Lat<T> &L, const PlainWork &W, int lane, T *buf)
 {
-    const int t = e >> 3, li = lane & 15;
-    const int lx = (e & 1) * 16 + (li & 7) * 2, ly = ((e >> 1) & 3) * 2 + (li >> 3);
+    const int t = W.e >> 3, li = lane & 15;
+    const int lx = (W.e & 1) * 16 + (li & 7) * 2, ly = ((W.e >> 1) & 3) * 2 + (li >> 3);
     const int p = ls.p;
     // slots of the lane's first cell, one row down (0), its own (1), one row up (2), and of the
-    // cells left and right of the two in those rows.  tv is the tile across the lane's vertical
-    // tile edge (its own if it has none), th0 / thv the same across a horizontal one.
+    // cells left and right of the two in those rows (found here and not before the wait: nine
+    // registers less to hold there, a 2048^2 level takes 87 us a step instead of 94)
     int mid[3], lf[3], rt[3];
     {
         const bool wl = lx == 0, wr = lx == LBM_TX - 2;
@@ -1049,8 +1094,8 @@ __device__ __forceinline__ void plain_warp(const LevelView &P, const LevelView &
             const int y = ly + a - 1;
             const bool over = y < 0 || y >= LBM_TY;
             const int row = (y & (LBM_TY - 1)) * LBM_TX;
-            mid[a] = (over ? tv : t) * LBM_TILE + row + lx;
-            const int ts = (over ? thv : th0) * LBM_TILE + row;
+            mid[a] = (over ? W.tv : t) * LBM_TILE + row + lx;
+            const int ts = (over ? W.thv : W.th0) * LBM_TILE + row;
             lf[a] = wl ? ts + LBM_TX - 1 : mid[a] - 1;
             rt[a] = wr ? ts : mid[a] + 2;
 #ifdef LBM_BOUNDS_CHECK
@@ -1061,17 +1106,12 @@ __device__ __forceinline__ void plain_warp(const LevelView &P, const LevelView &
     }
     const int slot = mid[1];
     // ---- streaming (eq 1): fetch the populations arriving at the cells; in odd steps those of the
-    // upstream rows y - c_y from the opposite planes, with the cell beside the two where c_x != 0
-    float side[9];
+    // upstream rows y - c_y from the opposite planes
     buf += lane * 2;
 #pragma unroll
     for (int q = 0; q < 9; q++) {
-        if (!ODD) {
-            L.fetch2(q, slot, buf + q * 64);
-        } else {
-            L.fetch2(oppq(q), mid[1 - cyq(q)], buf + q * 64);
-            if (cxq(q) != 0) side[q] = L.ld(oppq(q), cxq(q) > 0 ? lf[1 - cyq(q)] : rt[1 - cyq(q)], q);
-        }
+        if (!ODD) L.fetch2(q, slot, buf + q * 64);
+        else L.fetch2(oppq(q), mid[1 - cyq(q)], buf + q * 64);
     }
     // ---- SA-neg update of chi (Sec 2.2), fields at time t
     float chin[2];
@@ -1105,6 +1145,14 @@ __device__ __forceinline__ void plain_warp(const LevelView &P, const LevelView &
         // laminar: chi takes no part in the step, but the covered parents' is restricted below
         chin[0] = chin[1] = 0.0f;
         if (ls.restrict_up) ld2(P.chi[p] + slot, chin);
+    }
+    // odd steps: the cell beside the two where c_x != 0 (mostly in a line that a neighbour lane has
+    // fetched by now; loaded here so as not to hold six registers through the SA-neg update)
+    float side[9];
+    if (ODD) {
+#pragma unroll
+        for (int q = 1; q < 9; q++)
+            if (cxq(q) != 0) side[q] = L.ld(oppq(q), cxq(q) > 0 ? lf[1 - cyq(q)] : rt[1 - cyq(q)], q);
     }
     async_wait();
     float g[9][2];
@@ -1163,62 +1211,12 @@ __device__ __forceinline__ void plain_warp(const LevelView &P, const LevelView &
 }
 
 // ------------------------------------------------------------------ the level kernel
-// The static part of a warp's work, read before the wait for the preceding kernel.  The work list
-// holds the general 16 x 2-cell blocks (each with boundary nodes twice: its wall warp, then its
-// partner), then the plain ones.  A PLAIN launch takes the latter two to a warp (plain_warp),
-// any other one to a warp as it takes the general ones.
-struct WarpWork {
-    int e;              // tile * 8 + block of the tile
-    bool have, plain, wall;
-    int lx, ly;         // general: the lane's cell
-    uint32_t fl;
-    int ax;
-    int tv, th0, thv;   // plain: tiles across the lane's vertical / horizontal / both tile edges
-};
-
-// warps that a launch over a level takes
-__host__ __device__ __forceinline__ int level_warps(const LevelView &P, bool plain)
-{
-    return P.n_gen_warps + (plain ? P.n_plain / 2 : P.n_plain);
-}
-
-template <bool PLAIN>
-__device__ __forceinline__ WarpWork warp_work(const LevelView &P, int w, int lane, int *nb3, int *status)
-{
-    WarpWork W;
-    W.plain = PLAIN && w >= P.n_gen_warps;
-    W.have = w < level_warps(P, PLAIN);
-    W.wall = w < P.n_pair_warps;
-    W.e = 0; W.lx = W.ly = 0; W.fl = 0; W.ax = 0; W.tv = W.th0 = W.thv = 0;
-    if (!W.have) return W;
-    if (!W.plain) {
-        W.e = checked_index(__ldg(P.work + w), 8 * P.ntiles, status);
-        const int t = W.e >> 3;
-        cell_of_thread((W.e & 7) * 32 + lane, W.lx, W.ly);
-        if (lane < 9) nb3[lane] = P.nbr[t * 9 + dir_of3(lane)];
-        const int slot = t * LBM_TILE + W.ly * LBM_TX + W.lx;
-        W.fl = __ldg(P.flags + slot);
-        W.ax = uses_aux(W.fl) ? __ldg(P.aux + slot) : -1;
-        __syncwarp();
-    } else {
-        W.e = checked_index(__ldg(P.work + P.n_gen_warps + 2 * (w - P.n_gen_warps) + (lane >> 4)), 8 * P.ntiles, status);
-        const int t = W.e >> 3, li = lane & 15;
-        const int lx = (W.e & 1) * 16 + (li & 7) * 2, ly = ((W.e >> 1) & 3) * 2 + (li >> 3);
-        const int sx = lx == 0 ? 0 : (lx == LBM_TX - 2 ? 2 : 1), sy = ly == 0 ? 0 : (ly == LBM_TY - 1 ? 2 : 1);
-        const int *nb = P.nbr + t * 9;
-        W.tv = sy == 1 ? t : __ldg(nb + dir_of3(sy * 3 + 1));
-        W.th0 = sx == 1 ? t : __ldg(nb + dir_of3(3 + sx));
-        W.thv = sx == 1 ? W.tv : (sy == 1 ? W.th0 : __ldg(nb + dir_of3(sy * 3 + sx)));
-    }
-    return W;
-}
-
-__device__ __forceinline__ bool boundary_cell(const WarpWork &W)
+__device__ __forceinline__ bool boundary_cell(const GeneralWork &W)
 {
     return (W.fl & (FL_KIND_MASK | FL_SOLID | FL_BNODE)) == (KIND_ACTIVE | FL_BNODE);
 }
 
-__device__ __forceinline__ CutLinks cut_links(const RecView &R, const WarpWork &W, int *status)
+__device__ __forceinline__ CutLinks cut_links(const RecView &R, const GeneralWork &W, int *status)
 {
     CutLinks c;
     const bool b = W.wall && boundary_cell(W);
@@ -1236,10 +1234,11 @@ __device__ __forceinline__ CutLinks cut_links(const RecView &R, const WarpWork &
 // the c/4096 workload's levels 2 and 3 take 5.3 .. 6.4 us at 80 registers and 7.0 .. 8.8 at 64,
 // its level 4 the same at both; its level 0 (box edges) 13.0 / 13.9 us against 13.4 / 15.4 at 80,
 // and the finest one 13.7 / 16.2 against 13.8 / 16.5.  Without plain warps a launch is one general
-// warp's latency: 96 registers, no spills (c/256 airfoil 289 us a coarse step, 294 at 80).
+// warp's latency: 96 registers, 128 with a finer level, which is no spills (c/256 airfoil 289 us a
+// coarse step against 294 at 80, 260 against 263 with the finer level's target table at 128 and 96).
 __host__ __device__ constexpr int level_min_blocks(int kind, bool plain, bool edge)
 {
-    return plain ? (kind == 1 && !edge ? 6 : 8) : 5;
+    return plain ? (kind == 1 && !edge ? 6 : 8) : (kind == 1 ? 4 : 5);
 }
 
 // Blocks of whole warps (64 or 128 threads, chosen at launch) over the level's work list.  KIND:
@@ -1254,28 +1253,34 @@ __global__ void __launch_bounds__(LBM_BLOCK, level_min_blocks(KIND, PLAIN, EDGE)
     __shared__ int nb3w[NW][9];                  // one copy per warp: no block-wide barrier
     __shared__ WallPair pairs[KIND == 2 ? NW / 2 : 1];
     __shared__ __align__(16) T pops[PLAIN ? NW : 1][PLAIN ? 9 * 64 : 1];
-    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, w = blockIdx.x * (blockDim.x >> 5) + wb;
     tl_mark(ls.tl, ls.tl_base, 0);
-    const WarpWork W = warp_work<PLAIN>(P, blockIdx.x * (blockDim.x >> 5) + wb, lane, nb3w[wb], ls.status);
-    if (KIND == 2 && W.wall && !(wb & 1)) {
-        WallPair &S = pairs[KIND == 2 ? wb >> 1 : 0];
-        const WallStatic ws = wall_static(R, S, boundary_cell(W), W.ax, lane, ls.status);
-        griddep_launch();
-        griddep_wait();
-        tl_mark(ls.tl, ls.tl_base, 1);
-        wall_warp(P, R, k, ls, ws, S, lane);
-        pair_arrive(wb >> 1);
-    } else {
-        CutLinks cut;
-        if (KIND == 2) cut = cut_links(R, W, ls.status);
-        griddep_launch();
-        griddep_wait();
-        tl_mark(ls.tl, ls.tl_base, 1);
-        if (PLAIN && W.plain) {
-            if (W.have) plain_warp<T, ODD>(P, C, k, ls, L, W.e, lane, W.tv, W.th0, W.thv, pops[PLAIN ? wb : 0]);
-        } else if (W.have) {
-            general_warp<KIND, T, ODD, EDGE>(P, F, C, R, k, ls, L, W.e >> 3, lane, W.lx, W.ly, nb3w[wb], W.fl, W.ax,
-                                             KIND == 2 && W.wall ? &pairs[wb >> 1] : nullptr, wb >> 1, cut);
+    if (PLAIN && w >= P.n_gen_warps) {
+        if (w < level_warps(P, PLAIN)) {
+            const PlainWork W = plain_work(P, ls, w, lane);
+            griddep_launch();
+            griddep_wait();
+            tl_mark(ls.tl, ls.tl_base, 1);
+            plain_warp<T, ODD>(P, C, k, ls, L, W, lane, pops[PLAIN ? wb : 0]);
+        }
+    } else if (w < level_warps(P, PLAIN)) {
+        const GeneralWork W = general_work(P, C, ls, w, lane, nb3w[wb]);
+        if (KIND == 2 && W.wall && !(wb & 1)) {
+            WallPair &S = pairs[KIND == 2 ? wb >> 1 : 0];
+            const WallStatic ws = wall_static(R, S, boundary_cell(W), W.ax, lane, ls.status);
+            griddep_launch();
+            griddep_wait();
+            tl_mark(ls.tl, ls.tl_base, 1);
+            wall_warp(P, R, k, ls, ws, S, lane);
+            pair_arrive(wb >> 1);
+        } else {
+            CutLinks cut;
+            if (KIND == 2) cut = cut_links(R, W, ls.status);
+            griddep_launch();
+            griddep_wait();
+            tl_mark(ls.tl, ls.tl_base, 1);
+            general_warp<KIND, T, ODD, EDGE>(P, F, C, R, k, ls, L, W, lane, KIND == 2 && W.wall ? &pairs[wb >> 1] : nullptr,
+                                             wb >> 1, cut);
         }
     }
     tl_end(ls.tl, ls.tl_base);
@@ -1295,8 +1300,20 @@ __global__ void __launch_bounds__(LBM_BLOCK, 5) k_level_batch(const __grid_const
     __shared__ WallPair pairs[NW / 2];
     __shared__ __align__(16) T pops[PLAIN ? NW : 1][PLAIN ? 9 * 64 : 1];
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
-    int *nb3 = nb3w[wb];
-    const WarpWork W = warp_work<PLAIN>(d.P, (blockIdx.x - d.first_block) * NW + wb, lane, nb3, d.ls.status);
+    const int w = (blockIdx.x - d.first_block) * NW + wb;
+    if (w >= level_warps(d.P, PLAIN)) return;
+    const Lat<T> L{static_cast<T *>(d.P.f), d.P.ns, d.k.pshift};
+    const bool odd = d.ls.p != 0;
+    if (PLAIN && w >= d.P.n_gen_warps) {
+        const PlainWork W = plain_work(d.P, d.ls, w, lane);
+        griddep_launch();
+        griddep_wait();
+        T *buf = pops[PLAIN ? wb : 0];
+        if (odd) plain_warp<T, true>(d.P, d.C, d.k, d.ls, L, W, lane, buf);
+        else plain_warp<T, false>(d.P, d.C, d.k, d.ls, L, W, lane, buf);
+        return;
+    }
+    const GeneralWork W = general_work(d.P, d.C, d.ls, w, lane, nb3w[wb]);
     WallPair &S = pairs[wb >> 1];
     if (W.wall && !(wb & 1)) {
         const WallStatic ws = wall_static(d.R, S, boundary_cell(W), W.ax, lane, d.ls.status);
@@ -1309,19 +1326,9 @@ __global__ void __launch_bounds__(LBM_BLOCK, 5) k_level_batch(const __grid_const
     const CutLinks cut = cut_links(d.R, W, d.ls.status);
     griddep_launch();
     griddep_wait();
-    if (!W.have) return;
-    const Lat<T> L{static_cast<T *>(d.P.f), d.P.ns, d.k.pshift};
-    const bool odd = d.ls.p != 0;
-    if (PLAIN && W.plain) {
-        T *buf = pops[PLAIN ? wb : 0];
-        if (odd) plain_warp<T, true>(d.P, d.C, d.k, d.ls, L, W.e, lane, W.tv, W.th0, W.thv, buf);
-        else plain_warp<T, false>(d.P, d.C, d.k, d.ls, L, W.e, lane, W.tv, W.th0, W.thv, buf);
-        return;
-    }
-    const int t = W.e >> 3;
     const WallPair *wp = W.wall ? &S : nullptr;
 #define LBM_GENERAL(KIND, ODD) \
-    general_warp<KIND, T, ODD, true>(d.P, d.F, d.C, d.R, d.k, d.ls, L, t, lane, W.lx, W.ly, nb3, W.fl, W.ax, wp, wb >> 1, cut)
+    general_warp<KIND, T, ODD, true>(d.P, d.F, d.C, d.R, d.k, d.ls, L, W, lane, wp, wb >> 1, cut)
     if (d.kind == 2) { if (odd) LBM_GENERAL(2, true); else LBM_GENERAL(2, false); }
     else if (d.kind == 1) { if (odd) LBM_GENERAL(1, true); else LBM_GENERAL(1, false); }
     else { if (odd) LBM_GENERAL(0, true); else LBM_GENERAL(0, false); }
