@@ -55,9 +55,9 @@ __device__ __forceinline__ void prolong_write(const LevelView &P, const LevelVie
     Stencil S;
 #pragma unroll
     for (int q = 0; q < 9; q++) {
-        S.chi[q] = __ldg(P.chi[p] + c.s[q]); S.ux[q] = __ldg(P.ux[p] + c.s[q]); S.uy[q] = __ldg(P.uy[p] + c.s[q]);
+        S.chi[q] = P.chi[p][c.s[q]]; S.ux[q] = P.ux[p][c.s[q]]; S.uy[q] = P.uy[p][c.s[q]];
     }
-    const float dr = __ldg(P.drho[p] + c.s[0]);
+    const float dr = P.drho[p][c.s[0]];
     float gcx, gcy, gux, guy, gvx, gvy;
     lsq_grad(S.chi, gcx, gcy); lsq_grad(S.ux, gux, guy); lsq_grad(S.uy, gvx, gvy);
 #pragma unroll

@@ -115,18 +115,15 @@ __device__ __forceinline__ int child_base(const LevelView &P, int t, int lx, int
 // FP32 and every store rounds to nearest, so the arithmetic is FP32 in all three forms.
 template <typename T> struct PopIO;
 template <> struct PopIO<float> {
-    static __device__ __forceinline__ float ld(const float *p) { return __ldg(p); }
-    static __device__ __forceinline__ float ldp(const float *p) { return *p; }
+    static __device__ __forceinline__ float ld(const float *p) { return *p; }
     static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
 };
 template <> struct PopIO<__half> {
-    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(__ldg(p)); }
-    static __device__ __forceinline__ float ldp(const __half *p) { return __half2float(*p); }
+    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(*p); }
     static __device__ __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v); }
 };
 template <> struct PopIO<__nv_bfloat16> {
-    static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
-    static __device__ __forceinline__ float ldp(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+    static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
@@ -155,10 +152,12 @@ __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;"
 
 // ------------------------------------------------------------------ programmatic dependent launch
 // The level-step kernels are launched with programmatic stream serialization: the next
-// kernel's blocks may be scheduled while this one drains.  Each kernel reads only the
-// static tile tables before griddep_wait(), which returns once the preceding kernel has
+// kernel's blocks may be scheduled while this one drains.  Each kernel reads only
+// static tables before griddep_wait(), which returns once the preceding kernel has
 // completed and its writes are visible; griddep_launch() lets the next kernel start
-// being scheduled as soon as every block of this one has begun.
+// being scheduled as soon as every block of this one has begun.  What a preceding kernel may
+// have written is read with ordinary loads: __ldg tells the compiler that the value never
+// changes, and it then moves the load up across the wait.
 __device__ __forceinline__ void griddep_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -882,7 +881,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
         const float *xc = P.chi[p], *xu = P.ux[p], *xv = P.uy[p];
 #pragma unroll
         for (int q = 0; q < 9; q++) {
-            S.chi[q] = __ldg(xc + nbs[q]); S.ux[q] = __ldg(xu + nbs[q]); S.uy[q] = __ldg(xv + nbs[q]);
+            S.chi[q] = xc[nbs[q]]; S.ux[q] = xu[nbs[q]]; S.uy[q] = xv[nbs[q]];
         }
     }
     float id2 = sa ? __ldg(P.inv_d2 + slot) : 0.0f;
@@ -924,7 +923,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
     // ---- SA-neg update of chi (Sec 2.2), fields at time t
     float chin = 0.0f;
     if (act) {
-        if (!sa) chin = __ldg(P.chi[p] + slot);
+        if (!sa) chin = P.chi[p][slot];
         else if (edge && (fl & FL_INLET)) chin = k.chi_inf;
         else chin = sa_update(S, id2, P.nu, k.sa_convection);
     }
@@ -1051,7 +1050,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
 
 __device__ __forceinline__ void ld2(const float *a, float v[2])
 {
-    const float2 m = __ldg(reinterpret_cast<const float2 *>(a));
+    const float2 m = *reinterpret_cast<const float2 *>(a);
     v[0] = m.x; v[1] = m.y;
 }
 __device__ __forceinline__ void st2(float *a, const float v[2]) { *reinterpret_cast<float2 *>(a) = make_float2(v[0], v[1]); }
@@ -1059,9 +1058,9 @@ __device__ __forceinline__ void st2(float *a, const float v[2]) { *reinterpret_c
 // Row of four values around a lane's two cells: the cell to the left, the two, the one to the right.
 __device__ __forceinline__ void row4(const float *a, int left, int mid, int right, float v[4])
 {
-    v[0] = __ldg(a + left);
+    v[0] = a[left];
     ld2(a + mid, v + 1);
-    v[3] = __ldg(a + right);
+    v[3] = a[right];
 }
 
 // One warp over two plain 16 x 2-cell blocks (every cell active, none with a wall, interface or
