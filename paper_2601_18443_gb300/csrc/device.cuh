@@ -138,7 +138,9 @@ struct SolveDesc {
 };
 struct BatchArgs {
     int n;               // solves in this launch
-    bool plain;          // as LevelTune::plain
+    int kind;            // the members' SolveDesc::kind where all take the same kind of step and the
+    bool odd, edge;      // same parity (odd; edge: level 0 of a box with edges), else -1
+    bool plain;          // as LevelTune::plain (not with kind -1)
     SolveDesc d[LBM_BATCH_MAX];
 };
 struct ProlongDesc {

@@ -334,6 +334,9 @@ static void flush_prolong(lbm_solver *s, cudaStream_t st, long long &nk)
 // 11.5 / 13.1.
 static bool plain_form(long warps, int sms) { return warps > 20 * (long)sms; }
 
+// what the level kernel does on a level: 2 finest with wall records, 1 with a finer level, 0 neither
+static int level_kind(const lbm_solver *s, int l) { return l == s->L - 1 ? (s->rec.n > 0 ? 2 : 0) : 1; }
+
 // warps of a block of the level kernel under a grid schedule
 static int block_warps(int sched) { return sched == LBM_SCHED_WARPS ? 2 : LBM_BLOCK / 32; }
 
@@ -1808,6 +1811,9 @@ struct lbm_batch {
     cudaEvent_t done = nullptr;
     std::vector<cudaEvent_t> ready;
     long long kernels_per_step = 0;
+    lbmdev::ProlongBatchArgs pend{};   // prolongations waiting for the next level-step launch
+    unsigned pend_grid = 0;
+    int pend_level = 0;
     std::string err;
 };
 
@@ -1817,22 +1823,34 @@ static lbm_status bfail(lbm_batch *b, lbm_status code, const std::string &msg)
     return code;
 }
 
+static void batch_flush(lbm_batch *b, cudaStream_t st, long long &nk)
+{
+    if (b->pend_grid) { lbmdev::launch_prolong_batch(st, b->pend, b->pend_grid, 1); nk++; }
+    b->pend.n = 0;
+    b->pend_grid = 0;
+}
+
 static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up, long long &nk)
 {
-    // prolongation of level l into the ghosts of l + 1, for the members that have l + 1
+    // prolongation of level l into the ghosts of l + 1, for the members that have l + 1.  As in a
+    // single solve it waits for the next level step and joins the prolongation of level l - 1
+    // where no member's reads what that one writes and the descriptors have room
     {
-        lbmdev::ProlongBatchArgs a;
-        a.n = 0;
-        a.tl = nullptr;
-        a.tl_base = 0;
-        unsigned grid = 0;
+        bool joins = b->pend.n > 0 && b->pend_level + 1 == l;
+        int more = 0;
+        for (lbm_solver *s : b->m)
+            if (l + 1 < s->L && s->lv[l].v.n_band > 0) {
+                more++;
+                joins = joins && s->prolong_indep[l];
+            }
+        if (!joins || b->pend.n + more > LBM_BATCH_MAX) batch_flush(b, st, nk);
+        if (more) b->pend_level = l;
         for (lbm_solver *s : b->m) {
             if (l + 1 >= s->L || s->lv[l].v.n_band <= 0) continue;
-            lbmdev::ProlongDesc &d = a.d[a.n++];
-            d.P = s->lv[l].v; d.F = s->lv[l + 1].v; d.p = s->parity[l]; d.first_block = (int)grid;
-            grid += lbmdev::prolong_blocks(s->lv[l].v);
+            lbmdev::ProlongDesc &d = b->pend.d[b->pend.n++];
+            d.P = s->lv[l].v; d.F = s->lv[l + 1].v; d.p = s->parity[l]; d.first_block = (int)b->pend_grid;
+            b->pend_grid += lbmdev::prolong_blocks(s->lv[l].v);
         }
-        if (grid) { lbmdev::launch_prolong_batch(st, a, grid, 1); nk++; }
     }
     if (l + 1 < b->Lmax) {
         batch_advance(b, st, l + 1, 0, nk);
@@ -1840,10 +1858,21 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
     }
     lbmdev::BatchArgs a;
     a.n = 0;
+    batch_flush(b, st, nk);
+    // one kind and parity for all members, or the form for any mix
     int warps = 0;
-    for (lbm_solver *s : b->m)
-        if (l < s->L) warps += s->lv[l].v.n_gen_warps + s->lv[l].v.n_plain;
-    a.plain = plain_form(warps, b->m[0]->k.sms);
+    a.kind = -2;
+    a.odd = a.edge = false;
+    for (lbm_solver *s : b->m) {
+        if (l >= s->L) continue;
+        const int kind = level_kind(s, l);
+        const bool odd = s->parity[l] != 0, edge = l == 0 && s->k.level0_edges;
+        if (a.kind == -2) { a.kind = kind; a.odd = odd; a.edge = edge; }
+        else if (a.kind != kind || a.odd != odd) a.kind = -1;
+        else a.edge = a.edge || edge;
+        warps += s->lv[l].v.n_gen_warps + s->lv[l].v.n_plain;
+    }
+    a.plain = a.kind >= 0 && plain_form(warps, b->m[0]->k.sms);
     unsigned grid = 0;
     for (lbm_solver *s : b->m) {
         if (l >= s->L) continue;
@@ -1863,7 +1892,7 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
         d.ls.status = s->d_status;
         d.ls.tl = nullptr;
         d.ls.tl_base = 0;
-        d.kind = d.ls.wall ? 2 : (d.ls.has_child ? 1 : 0);
+        d.kind = level_kind(s, l);
         d.first_block = (int)grid;
         grid += (unsigned)((d.P.n_gen_warps + (a.plain ? d.P.n_plain / 2 : d.P.n_plain) + LBM_BLOCK / 32 - 1) / (LBM_BLOCK / 32));
         s->parity[l] ^= 1;

@@ -1240,98 +1240,103 @@ __host__ __device__ constexpr int level_min_blocks(int kind, bool plain, bool ed
     return plain ? (kind == 1 && !edge ? 6 : 8) : (kind == 1 ? 4 : 5);
 }
 
-// Blocks of whole warps (64 or 128 threads, chosen at launch) over the level's work list.  KIND:
-// 0 no finer level, 1 with a finer level, 2 finest level with wall records; ODD: the parity of the
-// in-place population update; EDGE: level 0 of a box with edges.
+// Shared memory of a block of the level kernel.
+template <int KIND, typename T, bool PLAIN> struct LevelShared {
+    static constexpr int NW = LBM_BLOCK / 32;
+    int nb3[NW][9];                                       // one copy per warp: no block-wide barrier
+    WallPair pairs[KIND == 2 ? NW / 2 : 1];
+    alignas(16) T pops[PLAIN ? NW : 1][PLAIN ? 9 * 64 : 1];
+};
+
+// Warp w of a launch over a level, warp wb of its block.  KIND: 0 no finer level, 1 with a finer
+// level, 2 finest level with wall records; ODD: the parity of the in-place population update;
+// EDGE: level 0 of a box with edges (or of a mixed batch).
+template <int KIND, typename T, bool ODD, bool PLAIN, bool EDGE, bool TIMELINE>
+__device__ __forceinline__ void level_warp(const LevelView &P, const LevelView &F, const LevelView &C, const RecView &R,
+                                           const StepConsts &k, const LevelStep &ls, LevelShared<KIND, T, PLAIN> &S, int w,
+                                           int wb, int lane)
+{
+    auto wait = [&]() {
+        griddep_launch();
+        griddep_wait();
+        if (TIMELINE) tl_mark(ls.tl, ls.tl_base, 1);
+    };
+    if (w >= level_warps(P, PLAIN)) return;
+    const Lat<T> L{static_cast<T *>(P.f), P.ns, k.pshift};
+    if (PLAIN && w >= P.n_gen_warps) {
+        const PlainWork W = plain_work(P, ls, w, lane);
+        wait();
+        plain_warp<T, ODD>(P, C, k, ls, L, W, lane, S.pops[PLAIN ? wb : 0]);
+        return;
+    }
+    const GeneralWork W = general_work(P, C, ls, w, lane, S.nb3[wb]);
+    if (KIND == 2 && W.wall && !(wb & 1)) {
+        WallPair &wp = S.pairs[KIND == 2 ? wb >> 1 : 0];
+        const WallStatic ws = wall_static(R, wp, boundary_cell(W), W.ax, lane, ls.status);
+        wait();
+        wall_warp(P, R, k, ls, ws, wp, lane);
+        pair_arrive(wb >> 1);
+        return;
+    }
+    CutLinks cut;
+    if (KIND == 2) cut = cut_links(R, W, ls.status);
+    wait();
+    general_warp<KIND, T, ODD, EDGE>(P, F, C, R, k, ls, L, W, lane, KIND == 2 && W.wall ? &S.pairs[wb >> 1] : nullptr,
+                                     wb >> 1, cut);
+}
+
+// Blocks of whole warps (64 or 128 threads, chosen at launch) over the level's work list.
 template <int KIND, typename T, bool ODD, bool PLAIN, bool EDGE>
 __global__ void __launch_bounds__(LBM_BLOCK, level_min_blocks(KIND, PLAIN, EDGE))
     k_level(LevelView P, LevelView F, LevelView C, RecView R, StepConsts k, LevelStep ls)
 {
-    constexpr int NW = LBM_BLOCK / 32;
-    const Lat<T> L{static_cast<T *>(P.f), P.ns, k.pshift};
-    __shared__ int nb3w[NW][9];                  // one copy per warp: no block-wide barrier
-    __shared__ WallPair pairs[KIND == 2 ? NW / 2 : 1];
-    __shared__ __align__(16) T pops[PLAIN ? NW : 1][PLAIN ? 9 * 64 : 1];
-    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, w = blockIdx.x * (blockDim.x >> 5) + wb;
+    __shared__ LevelShared<KIND, T, PLAIN> S;
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
     tl_mark(ls.tl, ls.tl_base, 0);
-    if (PLAIN && w >= P.n_gen_warps) {
-        if (w < level_warps(P, PLAIN)) {
-            const PlainWork W = plain_work(P, ls, w, lane);
-            griddep_launch();
-            griddep_wait();
-            tl_mark(ls.tl, ls.tl_base, 1);
-            plain_warp<T, ODD>(P, C, k, ls, L, W, lane, pops[PLAIN ? wb : 0]);
-        }
-    } else if (w < level_warps(P, PLAIN)) {
-        const GeneralWork W = general_work(P, C, ls, w, lane, nb3w[wb]);
-        if (KIND == 2 && W.wall && !(wb & 1)) {
-            WallPair &S = pairs[KIND == 2 ? wb >> 1 : 0];
-            const WallStatic ws = wall_static(R, S, boundary_cell(W), W.ax, lane, ls.status);
-            griddep_launch();
-            griddep_wait();
-            tl_mark(ls.tl, ls.tl_base, 1);
-            wall_warp(P, R, k, ls, ws, S, lane);
-            pair_arrive(wb >> 1);
-        } else {
-            CutLinks cut;
-            if (KIND == 2) cut = cut_links(R, W, ls.status);
-            griddep_launch();
-            griddep_wait();
-            tl_mark(ls.tl, ls.tl_base, 1);
-            general_warp<KIND, T, ODD, EDGE>(P, F, C, R, k, ls, L, W, lane, KIND == 2 && W.wall ? &pairs[wb >> 1] : nullptr,
-                                             wb >> 1, cut);
-        }
-    }
+    level_warp<KIND, T, ODD, PLAIN, EDGE, true>(P, F, C, R, k, ls, S, blockIdx.x * (blockDim.x >> 5) + wb, wb, lane);
     tl_end(ls.tl, ls.tl_base);
 }
 
-// The batched form of k_level: block b belongs to the last solve whose first block is at most b;
-// its kind and the parity of its level select the body.  Per cell it runs the same code.
-template <typename T, bool PLAIN>
-__global__ void __launch_bounds__(LBM_BLOCK, 5) k_level_batch(const __grid_constant__ BatchArgs a)
+// The batched form of k_level: block b belongs to the last solve whose first block is at most b.
+__device__ __forceinline__ int batch_member(const BatchArgs &a)
 {
     int i = 0;
     for (int m = 1; m < a.n; m++)
         if (a.d[m].first_block <= (int)blockIdx.x) i = m;
-    const SolveDesc &d = a.d[i];
-    constexpr int NW = LBM_BLOCK / 32;
-    __shared__ int nb3w[NW][9];
-    __shared__ WallPair pairs[NW / 2];
-    __shared__ __align__(16) T pops[PLAIN ? NW : 1][PLAIN ? 9 * 64 : 1];
+    return i;
+}
+
+// ... where all members take the same kind of step of the same parity (the serving loop groups by
+// level count): the code and the registers of k_level.  With one kernel that selects the kind and
+// the parity per block (k_level_batch, all six bodies in it) eight 5-level polar requests took
+// 312 us a coarse step, this way 257 (with the prolongations grouped as in a single solve).
+template <int KIND, typename T, bool ODD, bool PLAIN, bool EDGE>
+__global__ void __launch_bounds__(LBM_BLOCK, level_min_blocks(KIND, PLAIN, EDGE))
+    k_level_group(const __grid_constant__ BatchArgs a)
+{
+    const SolveDesc &d = a.d[batch_member(a)];
+    __shared__ LevelShared<KIND, T, PLAIN> S;
     const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
-    const int w = (blockIdx.x - d.first_block) * NW + wb;
-    if (w >= level_warps(d.P, PLAIN)) return;
-    const Lat<T> L{static_cast<T *>(d.P.f), d.P.ns, d.k.pshift};
+    level_warp<KIND, T, ODD, PLAIN, EDGE, false>(d.P, d.F, d.C, d.R, d.k, d.ls, S,
+                                                 ((int)blockIdx.x - d.first_block) * (LBM_BLOCK / 32) + wb, wb, lane);
+}
+
+// ... and for any mix: the member's kind and parity select the body.
+template <typename T>
+__global__ void __launch_bounds__(LBM_BLOCK, 5) k_level_batch(const __grid_constant__ BatchArgs a)
+{
+    const SolveDesc &d = a.d[batch_member(a)];
+    __shared__ LevelShared<0, T, false> S0;
+    __shared__ LevelShared<1, T, false> S1;
+    __shared__ LevelShared<2, T, false> S2;
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, w = ((int)blockIdx.x - d.first_block) * (LBM_BLOCK / 32) + wb;
     const bool odd = d.ls.p != 0;
-    if (PLAIN && w >= d.P.n_gen_warps) {
-        const PlainWork W = plain_work(d.P, d.ls, w, lane);
-        griddep_launch();
-        griddep_wait();
-        T *buf = pops[PLAIN ? wb : 0];
-        if (odd) plain_warp<T, true>(d.P, d.C, d.k, d.ls, L, W, lane, buf);
-        else plain_warp<T, false>(d.P, d.C, d.k, d.ls, L, W, lane, buf);
-        return;
-    }
-    const GeneralWork W = general_work(d.P, d.C, d.ls, w, lane, nb3w[wb]);
-    WallPair &S = pairs[wb >> 1];
-    if (W.wall && !(wb & 1)) {
-        const WallStatic ws = wall_static(d.R, S, boundary_cell(W), W.ax, lane, d.ls.status);
-        griddep_launch();
-        griddep_wait();
-        wall_warp(d.P, d.R, d.k, d.ls, ws, S, lane);
-        pair_arrive(wb >> 1);
-        return;
-    }
-    const CutLinks cut = cut_links(d.R, W, d.ls.status);
-    griddep_launch();
-    griddep_wait();
-    const WallPair *wp = W.wall ? &S : nullptr;
-#define LBM_GENERAL(KIND, ODD) \
-    general_warp<KIND, T, ODD, true>(d.P, d.F, d.C, d.R, d.k, d.ls, L, W, lane, wp, wb >> 1, cut)
-    if (d.kind == 2) { if (odd) LBM_GENERAL(2, true); else LBM_GENERAL(2, false); }
-    else if (d.kind == 1) { if (odd) LBM_GENERAL(1, true); else LBM_GENERAL(1, false); }
-    else { if (odd) LBM_GENERAL(0, true); else LBM_GENERAL(0, false); }
-#undef LBM_GENERAL
+#define LBM_BATCH_BODY(KIND, ODD) \
+    level_warp<KIND, T, ODD, false, true, false>(d.P, d.F, d.C, d.R, d.k, d.ls, S##KIND, w, wb, lane)
+    if (d.kind == 2) { if (odd) LBM_BATCH_BODY(2, true); else LBM_BATCH_BODY(2, false); }
+    else if (d.kind == 1) { if (odd) LBM_BATCH_BODY(1, true); else LBM_BATCH_BODY(1, false); }
+    else { if (odd) LBM_BATCH_BODY(0, true); else LBM_BATCH_BODY(0, false); }
+#undef LBM_BATCH_BODY
 }
 
 // ------------------------------------------------------------------ launchers
@@ -1391,10 +1396,30 @@ void launch_level_store(cudaStream_t st, const LevelView &P, const LevelView &Fv
     else launch_level_t<T, false>(st, P, Fv, Cv, child, R, k, ls, tu);
 }
 
+template <typename T, bool ODD, bool PLAIN, bool EDGE>
+static void launch_group_e(cudaStream_t st, const BatchArgs &a, unsigned grid, int pdl)
+{
+    if (a.kind == 2) launch_pdl_bs(k_level_group<2, T, ODD, PLAIN, EDGE>, grid, LBM_BLOCK, st, pdl, a);
+    else if (a.kind == 1) launch_pdl_bs(k_level_group<1, T, ODD, PLAIN, EDGE>, grid, LBM_BLOCK, st, pdl, a);
+    else launch_pdl_bs(k_level_group<0, T, ODD, PLAIN, EDGE>, grid, LBM_BLOCK, st, pdl, a);
+}
+
+template <typename T, bool ODD> static void launch_group(cudaStream_t st, const BatchArgs &a, unsigned grid, int pdl)
+{
+    if (a.plain) {
+        if (a.edge) launch_group_e<T, ODD, true, true>(st, a, grid, pdl);
+        else launch_group_e<T, ODD, true, false>(st, a, grid, pdl);
+    } else {
+        if (a.edge) launch_group_e<T, ODD, false, true>(st, a, grid, pdl);
+        else launch_group_e<T, ODD, false, false>(st, a, grid, pdl);
+    }
+}
+
 template <typename T> void launch_level_batch_store(cudaStream_t st, const BatchArgs &a, unsigned grid, int pdl)
 {
-    if (a.plain) launch_pdl_bs(k_level_batch<T, true>, grid, LBM_BLOCK, st, pdl, a);
-    else launch_pdl_bs(k_level_batch<T, false>, grid, LBM_BLOCK, st, pdl, a);
+    if (a.kind < 0) launch_pdl_bs(k_level_batch<T>, grid, LBM_BLOCK, st, pdl, a);
+    else if (a.odd) launch_group<T, true>(st, a, grid, pdl);
+    else launch_group<T, false>(st, a, grid, pdl);
 }
 
 }  // namespace lbmdev
