@@ -835,7 +835,7 @@ __device__ __forceinline__ void wall_warp(const LevelView &P, const RecView &R, 
 // thread and the boundary nodes' work in line, 2.8 / 3.2 us this way; level 4 (interfaces on both
 // sides) 4.9 / 6.6 us, then 3.3 / 4.6 with neighbour slots, parents and the explosion's targets
 // found after the wait, now 2.6 / 3.3 us.
-template <int KIND, typename T, bool ODD, bool EDGE>
+template <int KIND, typename T, bool ODD, bool PLAIN, bool EDGE>
 __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView &F, const LevelView &C, const RecView &R,
                                              const StepConsts &k, const LevelStep &ls, const Lat<T> &L, const GeneralWork &W,
                                              int lane, const WallPair *wp, int pair, const CutLinks &cut)
@@ -875,6 +875,12 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
 #pragma unroll
         for (int q = 0; q < 9; q++) x[q] = sb ? sb[q] : 0.0f;
     }
+    const bool band = CHILD && act && (fl & FL_BAND);
+    if (CHILD && act && (fl & (FL_BAND | (0xFFu << FL_COAL_SHIFT)))) ax = checked_index(ax, P.n_band, ls.status);
+    // the explosion's targets: with the first round of loads where the registers allow it (launches
+    // without plain warps), else behind the SA-neg update
+    BandTargets tgt = {};
+    if (!PLAIN && band) tgt = band_targets(P, ax);
     Stencil S;
     const bool sa = k.turbulence != 0 && __any_sync(0xffffffffu, act);
     if (sa) {
@@ -885,6 +891,9 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
         }
     }
     float id2 = sa ? __ldg(P.inv_d2 + slot) : 0.0f;
+    // (keeps the compiler from moving the stencil's loads down to their use, behind the branches
+    // below and the loads that they wait for)
+    asm volatile("" ::: "memory");
     int gi = 0, gj = 0;
     if (edge) {
         gi = P.tile_x[t] * LBM_TX + lx; gj = P.tile_y[t] * LBM_TY + ly;
@@ -905,8 +914,6 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
             }
         }
     }
-    const bool band = CHILD && act && (fl & FL_BAND);
-    if (CHILD && act && (fl & (FL_BAND | (0xFFu << FL_COAL_SHIFT)))) ax = checked_index(ax, P.n_band, ls.status);
     if (CHILD && (fl & (0xFFu << FL_COAL_SHIFT)) && act) {
         // coalescence: mean of what the four ghost children pulled in the fine level's odd sub-step
         const float4 *gb = reinterpret_cast<const float4 *>(P.gbuf + ax * 36);
@@ -927,8 +934,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
         else if (edge && (fl & FL_INLET)) chin = k.chi_inf;
         else chin = sa_update(S, id2, P.nu, k.sa_convection);
     }
-    BandTargets tgt = {};
-    if (band) tgt = band_targets(P, ax);
+    if (PLAIN && band) tgt = band_targets(P, ax);
     // ---- wall function of the boundary nodes (Sec 2.3), fields at time t, from the partner warp
     // (all lanes wait, whatever their cells)
     float drW = 0.f, uWx = 0.f, uWy = 0.f;
@@ -1281,7 +1287,7 @@ __device__ __forceinline__ void level_warp(const LevelView &P, const LevelView &
     CutLinks cut;
     if (KIND == 2) cut = cut_links(R, W, ls.status);
     wait();
-    general_warp<KIND, T, ODD, EDGE>(P, F, C, R, k, ls, L, W, lane, KIND == 2 && W.wall ? &S.pairs[wb >> 1] : nullptr,
+    general_warp<KIND, T, ODD, PLAIN, EDGE>(P, F, C, R, k, ls, L, W, lane, KIND == 2 && W.wall ? &S.pairs[wb >> 1] : nullptr,
                                      wb >> 1, cut);
 }
 
