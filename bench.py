@@ -13,7 +13,7 @@ Arms:
   default            the CUDA library (one replica per rank under torchrun, no collective)
   --impl reference   the FP64 CPU oracle on the host cores (rank 0 only)
 
-Launch variant: lbm_autotune picks each level's register budget and PDL on/off from timed
+Launch variant: lbm_autotune picks each level's warps per block and PDL on/off from timed
 steps before the warm-up (--no-autotune keeps the default variant).
 
 Timing: W untimed warm-up steps, then K steps timed with CUDA events on the solver's
@@ -57,9 +57,9 @@ def ncu_traffic(key):
                 if ln.strip() and not ln.startswith("#"):
                     k, v = ln.split()
                     vals[k] = v
-        src = os.path.join(ROOT, "paper_2601_18443_gb300", "csrc", "kernels.cu")
+        src = os.path.join(ROOT, "paper_2601_18443_gb300", "csrc", "level.cuh")
         with open(src, "rb") as f:
-            if hashlib.sha256(f.read()).hexdigest() != vals["kernels_cu_sha256"]:
+            if hashlib.sha256(f.read()).hexdigest() != vals["level_cuh_sha256"]:
                 return None
         return int(vals[key])
     except Exception:
@@ -69,8 +69,9 @@ def ncu_traffic(key):
 def method_bytes(store, turbulence):
     """Algorithmic bytes of the method per node update: the stream-collide moves 9 populations
     in and out, reads chi and writes rho and u (88 B in FP32, 52 B with 16-bit storage); SA-neg
-    adds chi read and written, u and 1/d^2 read (20 B).  The kernel also reads each cell's
-    flag word, which lbm_get_info counts in its bytes_per_node_update."""
+    adds chi read and written, u and 1/d^2 read (20 B).  The general form of the
+    kernel also reads each cell's flag word, which lbm_get_info counts in its
+    bytes_per_node_update; blocks of plain cells read no flag word and, laminar, no chi."""
     pop = 4 if store == 0 else 2
     return 18 * pop + 4 + 12 + (20 if turbulence else 0)
 
@@ -322,7 +323,7 @@ def gpu_arm(args, rank, world, dist):
     K = args.steps
     s = pkg.Solver(cfg, stream=stream)
     s.set_geometry(loops)
-    # launch autotuner (per-level register budget, grid schedule, work shape, PDL on/off);
+    # launch autotuner (warps per block of each level, PDL on/off);
     # its steps are untimed
     if args.no_autotune:
         tune = None
@@ -557,14 +558,16 @@ def hbm_grid_roofline(pkg, stream, peak, peak_kind, n=4096, turbulence=1, tune=T
     cells = info["cells_active"][0]
     bpn = method_bytes(store, turbulence)
     bpl = cells * bpn
+    # every block of the periodic level is plain: no flag word, and chi only with SA-neg
+    bpk = info["bytes_per_node_update"] - (4 if turbulence else 8)
     s.close()
     ach = bpl / (avg * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": round(ach, 1), "peak": peak, "unit": "GB/s", "frac": round(ach / peak, 4),
             "traffic": (ncu_traffic("hbm_grid_launch" if turbulence else "stream_collide_launch") if not store else None),
             "kernel": "k_level", "grid": f"{n}x{n} periodic, 1 level, SA {'on' if turbulence else 'off'}",
             "bytes_per_node_update": bpn, "bytes_per_launch": int(bpl),
-            "kernel_bytes_per_node_update": info["bytes_per_node_update"],
-            "frac_kernel_bytes": round(cells * info["bytes_per_node_update"] / (avg * 1e-3) / 1e9 / peak, 4),
+            "kernel_bytes_per_node_update": bpk,
+            "frac_kernel_bytes": round(cells * bpk / (avg * 1e-3) / 1e9 / peak, 4),
             "avg_launch_ms": round(avg, 4), "mlups": round(cells / avg / 1e3, 1),
             "peak_kind": peak_kind}
 
@@ -710,8 +713,8 @@ def main():
     ap.add_argument("--timeline", action="store_true",
                     help="profile case: also print the in-graph launch times (lbm_get_timeline) per level")
     ap.add_argument("--profile-variant", default="",
-                    help="profile case: launch variant 'min_blocks,sched,shape' on every level (sched 0 tile "
-                         "blocks, 1 persistent grid, 2 warp list) instead of autotuning")
+                    help="profile case: launch variant 'min_blocks,sched,shape' on every level (sched 2 two-warp "
+                         "blocks, otherwise four-warp blocks) instead of autotuning")
     ap.add_argument("--workload", choices=["naca0012", "highlift"], default="naca0012",
                     help="highlift: the three-element 8-level case (10 timed steps, no extra measurements)")
     ap.add_argument("--serving", type=int, default=0, help="serve this many requests of the polar stream")

@@ -89,7 +89,8 @@ typedef struct {
     long long wall_records, cut_links, surface_segments;
     long long kernels_per_step;   /* kernel launches issued per coarse step                          */
     double bytes_per_node_update; /* bytes the fused level step moves per node update (populations, flag
-                                     word, chi, rho and u; with SA-neg also chi written, u and 1/d^2 read) */
+                                     word, chi, rho and u; with SA-neg also chi written, u and 1/d^2 read;
+                                     blocks of plain cells read no flag word and, laminar, no chi) */
     double device_bytes;          /* device memory held by the handle                                */
     long long work_tiles[16];     /* tiles per level holding an active or ghost fluid cell           */
     long long work_warps[16];     /* 16 x 2-cell warps of those tiles that hold one                   */
