@@ -747,13 +747,19 @@ struct WallPair {
 // constant in each branch: with a number from a register the block would reserve all 16 barriers,
 // which leaves room for four blocks per SM (the c/4096 workload's finest level: 17.7 / 21.2 us for
 // its even / odd step that way, 13.8 / 16.5 us this way).
+// Both instructions are the aligned forms, which all lanes of a warp must execute together, and
+// they order memory between the warps only for what each lane wrote before.  What precedes them
+// branches per lane (the Newton iteration's length, the lanes that hold a result), so each first
+// brings its warp's lanes together.
 __device__ __forceinline__ void pair_arrive(int pair)
 {
+    __syncwarp();
     if (pair == 0) asm volatile("bar.arrive 1, 64;" ::: "memory");
     else asm volatile("bar.arrive 2, 64;" ::: "memory");
 }
 __device__ __forceinline__ void pair_wait(int pair)
 {
+    __syncwarp();
     if (pair == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
     else asm volatile("bar.sync 2, 64;" ::: "memory");
 }
@@ -939,7 +945,6 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
     // (all lanes wait, whatever their cells)
     float drW = 0.f, uWx = 0.f, uWy = 0.f;
     if (WALL && wp) {
-        __syncwarp();
         pair_wait(pair);
         if (bnode) {
             const float4 w = wp->res[lane];
