@@ -185,7 +185,10 @@ lbm_status lbm_get_level_box(lbm_solver *s, int level, int *i0, int *j0, int *nx
  * element capacity of each array (>= nx * ny).  rho, ux, uy in lattice units; nu_tilde_ratio
  * is nu_tilde / nu (chi).  Cells without values hold NaN.  mask: 0 absent, 1 active fluid,
  * 2 boundary node B, 3 covered, 4 ghost, 5 solid.  On a host-only handle only the mask
- * may be requested (LBM_ERR_NO_GEOMETRY otherwise). */
+ * may be requested (LBM_ERR_NO_GEOMETRY otherwise).  Calls on one handle may overlap from
+ * several threads, as long as no call that changes the handle's state (a step, lbm_set_*)
+ * overlaps them.  The handle keeps one host buffer of 16 bytes a slot of the largest level
+ * read (lbm_info.slots) until its grid is freed. */
 lbm_status lbm_get_fields(lbm_solver *s, int level, double *rho, double *ux, double *uy,
                           double *nu_tilde_ratio, unsigned char *mask, int cap);
 

@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -128,7 +129,8 @@ struct lbm_solver {
     cudaGraphExec_t bulk[2] = {nullptr, nullptr};    // bulk_steps() coarse steps, captured when first needed
     bool bulk_off = false;         // a bulk capture failed
     std::vector<void *> allocs;
-    lbmgrid::cellvec<float> host_fields;   // fields of a level on their way to the caller (download_level)
+    std::mutex host_m;                     // guards host_spare
+    lbmgrid::cellvec<float> host_spare;    // host buffer for a level's fields while no call uses it (FieldBuffer)
     double device_bytes = 0;
     int *d_status = nullptr;
     double *d_acc = nullptr;
@@ -239,7 +241,10 @@ static void free_all(lbm_solver *s)
         else cudaFree(p);
     }
     s->allocs.clear();
-    lbmgrid::cellvec<float>().swap(s->host_fields);
+    {
+        std::lock_guard<std::mutex> lock(s->host_m);
+        lbmgrid::cellvec<float>().swap(s->host_spare);
+    }
     s->device_bytes = 0;
     s->geometry = false;
     s->d_tl = nullptr;
@@ -1232,21 +1237,43 @@ lbm_status lbm_get_level_box(lbm_solver *s, int level, int *i0, int *j0, int *nx
     return LBM_OK;
 }
 
-// rho - 1, u_x, u_y, chi of a level at the current time into the handle's host buffer, one after
-// the other (v.ns values each).  The buffer is kept with the handle, sized for the largest level
-// asked for: copies into memory touched before run at 176 GB/s here, into fresh pages at 6 .. 18.
-static lbm_status download_level(lbm_solver *s, int l, float **out)
+// A call's own host buffer for a level's fields.  The handle keeps one buffer between calls, since
+// copies into memory touched before run at 176 GB/s here and into fresh pages at 6 .. 18.  A call
+// takes it with it, one that overlaps it on another thread allocates its own, and the larger of
+// the two stays when they end: at most one buffer, of the largest level asked for.
+struct FieldBuffer {
+    lbm_solver *s;
+    lbmgrid::cellvec<float> v;
+    explicit FieldBuffer(lbm_solver *solver) : s(solver)
+    {
+        std::lock_guard<std::mutex> lock(s->host_m);
+        v.swap(s->host_spare);
+    }
+    ~FieldBuffer()
+    {
+        std::lock_guard<std::mutex> lock(s->host_m);
+        if (v.size() > s->host_spare.size()) v.swap(s->host_spare);
+    }
+    FieldBuffer(const FieldBuffer &) = delete;
+    FieldBuffer &operator=(const FieldBuffer &) = delete;
+};
+
+// rho - 1, u_x, u_y, chi of a level at the current time into the buffer, one after the other
+// (v.ns values each).
+static lbm_status download_level(lbm_solver *s, int l, FieldBuffer &buf)
 {
     const LevelView &v = s->lv[l].v;
     const size_t n = 4 * (size_t)v.ns;
     try {
-        if (s->host_fields.size() < n) s->host_fields.resize(n);
+        if (buf.v.size() < n) {
+            buf.v.clear();                      // (nothing to move into the larger block)
+            buf.v.resize(n);
+        }
     } catch (const std::bad_alloc &) {
         return fail(s, LBM_ERR_OOM, "host memory for the fields");
     }
-    CK(cudaMemcpyAsync(s->host_fields.data(), v.drho[s->parity[l]], n * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(buf.v.data(), v.drho[s->parity[l]], n * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    *out = s->host_fields.data();
     return LBM_OK;
 }
 
@@ -1269,11 +1296,12 @@ lbm_status lbm_get_fields(lbm_solver *s, int level, double *rho, double *ux, dou
     if ((long long)nx * ny > cap) return fail(s, LBM_ERR_INVALID_ARG, "capacity too small");
     const bool fields = rho || ux || uy || chi;
     if (fields && !s->geometry) return fail(s, LBM_ERR_NO_GEOMETRY, "no device state (host-only handle): only the mask");
-    float *f = nullptr;
+    FieldBuffer buf(s);
     if (fields) {
-        st = download_level(s, level, &f);
+        st = download_level(s, level, buf);
         if (st != LBM_OK) return st;
     }
+    const float *f = buf.v.data();
     const lbmgrid::Level &G = s->g.lv[level];
     const size_t ns = (size_t)s->lv[level].v.ns;
     // rows in parallel, a row in pieces of one tile (consecutive slots): converting and placing the
@@ -1408,9 +1436,10 @@ lbm_status lbm_set_fields(lbm_solver *s, int level, const double *rho, const dou
     const LevelView &v = s->lv[level].v;
     const int p = s->parity[level];
     std::vector<float> c3(v.ns), post;
-    float *f = nullptr;
-    st = download_level(s, level, &f);
+    FieldBuffer buf(s);
+    st = download_level(s, level, buf);
     if (st != LBM_OK) return st;
+    float *f = buf.v.data();
     float *dr = f, *u = f + v.ns, *w = f + 2 * (size_t)v.ns, *c2 = f + 3 * (size_t)v.ns;
     CK(cudaMemcpyAsync(c3.data(), v.chi[p ^ 1], v.ns * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
     if ((st = gather_post(s, level, post)) != LBM_OK) return st;
