@@ -128,6 +128,7 @@ struct lbm_solver {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // one coarse step, by level-0 parity
     cudaGraphExec_t bulk[2] = {nullptr, nullptr};    // bulk_steps() coarse steps, captured when first needed
     bool bulk_off = false;         // a bulk capture failed
+    long long single_steps = 0;    // steps taken one by one since the graphs were captured
     std::vector<void *> allocs;
     std::mutex host_m;                     // guards host_spare
     lbmgrid::cellvec<float> host_spare;    // host buffer for a level's fields while no call uses it (FieldBuffer)
@@ -415,6 +416,7 @@ static lbm_status capture_graphs(lbm_solver *s)
 {
     s->tl_next = 0;
     s->tl_meta.clear();
+    s->single_steps = 0;
     for (int b = 0; b < 2; b++) {
         if (s->graph[b]) { cudaGraphExecDestroy(s->graph[b]); s->graph[b] = nullptr; }
         if (s->bulk[b]) { cudaGraphExecDestroy(s->bulk[b]); s->bulk[b] = nullptr; }
@@ -436,14 +438,15 @@ static lbm_status capture_graphs(lbm_solver *s)
 // Coarse steps of a bulk graph (an even number, so that it leaves the parity as it was), or 0
 // where there is none.  A graph launch takes about 6 us of host time and between two graphs the
 // next kernel is not scheduled while the last drains, so solves of few launches a step, whose
-// steps are as short as that, take eight steps a graph: 300 steps of a 1003 x 517 tunnel and a
-// read of its fields 5.36 -> 4.27 ms, 20 steps of a 64 x 40 box 279 -> 211 us, 100 steps of a
-// 4-level polar request (19 launches a step, two steps a graph) 8.67 -> 8.51 ms.
-// From 33 launches a step on that is under 1 % of the step.  With the timeline on every step goes
-// through the single-step graphs, which hold its records.
+// steps are as short as that, take up to eight steps a graph: 300 steps of a 1003 x 517 tunnel and
+// a read of its fields 5.36 -> 4.27 ms, 128 steps of a 64 x 40 box 806 -> 351 us, of two levels
+// (4 launches a step) 2120 -> 1513, of three (9 launches) 3784 -> 3564.  A 4-level polar request
+// (19 launches, two steps a graph) takes 8.50 ms for 128 steps one by one and 8.54 in bulk: the
+// line lies between.  With the timeline on every step goes through the single-step graphs, which
+// hold its records.
 static int bulk_steps(const lbm_solver *s)
 {
-    if (s->tl_on || s->bulk_off || s->kernels_per_step < 1 || s->kernels_per_step > 32) return 0;
+    if (s->tl_on || s->bulk_off || s->kernels_per_step < 1 || s->kernels_per_step > 16) return 0;
     return (int)std::min(8LL, 64 / s->kernels_per_step) & ~1;
 }
 
@@ -461,6 +464,16 @@ static bool have_bulk(lbm_solver *s, int nb)
     return false;
 }
 
+// Whether the steps that are left are to go through the bulk graph.  Its capture takes the host
+// 40, 120 and 180 us with 1, 4 and 9 launches a step and saves 3.5, 4.7 and 1.7 us of each step
+// after it, which is repaid after 11, 25 and 106 steps.  So it is made once the steps since the
+// single-step graphs were captured, with those left now, reach about that many: a handle's first
+// call of 8 steps takes 78, 160 and 278 us one by one, 83, 238 and 431 with the capture in it.
+static bool bulk_pays(const lbm_solver *s, int left)
+{
+    return s->bulk[s->parity[0]] || s->single_steps + left >= 4 + 12 * s->kernels_per_step;
+}
+
 static lbm_status enqueue_mass(lbm_solver *s);
 static void enqueue_history(lbm_solver *s);
 
@@ -470,7 +483,7 @@ static lbm_status enqueue_steps(lbm_solver *s, int n)
     for (int it = 0; it < n;) {
         // steps up to the next record of the load history, in bulk where they suffice
         const int left = s->hist_every > 0 ? std::min(n - it, (int)(s->hist_every - s->step % s->hist_every)) : n - it;
-        if (nb > 0 && left >= nb && !s->bulk_off && have_bulk(s, nb)) {
+        if (nb > 0 && left >= nb && !s->bulk_off && bulk_pays(s, left) && have_bulk(s, nb)) {
             CK(cudaGraphLaunch(s->bulk[s->parity[0]], s->stream));
             s->step += nb;
             it += nb;
@@ -478,6 +491,7 @@ static lbm_status enqueue_steps(lbm_solver *s, int n)
             CK(cudaGraphLaunch(s->graph[s->parity[0]], s->stream));
             s->parity[0] ^= 1;
             s->step++;
+            s->single_steps++;
             it++;
         }
         if (s->hist_every > 0 && s->step % s->hist_every == 0) enqueue_history(s);
