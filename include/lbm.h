@@ -407,7 +407,8 @@ lbm_status lbm_get_timeline(lbm_solver *s, lbm_launch_time *out, int cap, int *n
 /* Launch grouping of the prolongations (Sec 2.1): in each descent of the recursive schedule
  * the prolongations of consecutive levels l - 1, l go out as one launch (on by default)
  * where level l's band cells have no ghost cell of level l in their 3 x 3 neighbourhood, so
- * that neither reads what the other writes.  on 0 launches each on its own.  merged_levels
+ * that neither reads what the other writes.  on 0 launches each on its own, and so does a batch
+ * created later with the handle among its members.  merged_levels
  * (may be NULL) returns the number of levels l whose prolongation can join the one of
  * l - 1.  The step graphs are recaptured.  No device work.  Errors: LBM_ERR_INVALID_ARG,
  * LBM_ERR_NO_GEOMETRY. */

@@ -1893,14 +1893,15 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
 {
     // prolongation of level l into the ghosts of l + 1, for the members that have l + 1.  As in a
     // single solve it waits for the next level step and joins the prolongation of level l - 1
-    // where no member's reads what that one writes and the descriptors have room
+    // where every member groups its own (lbm_set_prolong_merge), none reads what that one writes and
+    // the descriptors have room
     {
         bool joins = b->pend.n > 0 && b->pend_level + 1 == l;
         int more = 0;
         for (lbm_solver *s : b->m)
             if (l + 1 < s->L && s->lv[l].v.n_band > 0) {
                 more++;
-                joins = joins && s->prolong_indep[l];
+                joins = joins && s->prolong_merge && s->prolong_indep[l];
             }
         if (!joins || b->pend.n + more > LBM_BATCH_MAX) batch_flush(b, st, nk);
         if (more) b->pend_level = l;
