@@ -127,7 +127,7 @@ struct lbm_solver {
     bool off_schedule = false;    // single launches (lbm_step_launch) left the level schedule
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // one coarse step, by level-0 parity
     cudaGraphExec_t bulk[2] = {nullptr, nullptr};    // bulk_steps() coarse steps, captured when first needed
-    bool bulk_off = false;         // a bulk capture failed
+    bool bulk_off = false;         // a bulk capture failed since the graphs were captured
     long long single_steps = 0;    // steps taken one by one since the graphs were captured
     std::vector<void *> allocs;
     std::mutex host_m;                     // guards host_spare
@@ -417,6 +417,7 @@ static lbm_status capture_graphs(lbm_solver *s)
     s->tl_next = 0;
     s->tl_meta.clear();
     s->single_steps = 0;
+    s->bulk_off = false;                    // (a later capture may find the memory, a new grid needs less)
     for (int b = 0; b < 2; b++) {
         if (s->graph[b]) { cudaGraphExecDestroy(s->graph[b]); s->graph[b] = nullptr; }
         if (s->bulk[b]) { cudaGraphExecDestroy(s->bulk[b]); s->bulk[b] = nullptr; }
