@@ -302,10 +302,11 @@ lbm_status lbm_time_kernels(lbm_solver *s, int n_coarse_steps, lbm_kernel_times 
  * lbm_set_launch_variant for callers that hold saved variants.
  * The choice comes from per-launch CUDA-event timings of `steps` eager
  * coarse steps per candidate, and is kept only if `steps` coarse steps through the step
- * graphs confirm it (against the same choice with LBM_SCHED_TILE where it picked
- * LBM_SCHED_PERSIST, against the form before tuning, and against each candidate on every
- * level; the fastest of these is kept), since launches overlap inside the
- * graphs.  Then it picks whether launches use programmatic dependent launch, from the time
+ * graphs confirm it (against the form before tuning and against each candidate on every
+ * level), since launches overlap inside the graphs.  Candidates with the same warps per block
+ * are the same launches: they count as one form with the median of their times, which goes by
+ * the first of them in the report.
+ * Then it picks whether launches use programmatic dependent launch, from the time
  * of `steps` coarse steps through the step graphs each way, and recaptures the graphs with
  * the choice.  The variants compute the same numbers up to FP32 rounding (the compiler
  * schedules and contracts the arithmetic differently per variant); the timed steps are real
@@ -321,10 +322,10 @@ typedef struct {
     int min_blocks[16];                       /* chosen min_blocks per level                       */
     int sched[16];                            /* chosen grid schedule per level (LBM_SCHED_*)      */
     int shape[16];                            /* chosen work shape per level                       */
-    double step_us_confirm[3 + LBM_TUNE_CANDIDATES]; /* coarse step: per-level pick, pick with
-                                                 TILE for PERSIST, form before
+    double step_us_confirm[3 + LBM_TUNE_CANDIDATES]; /* coarse step: per-level pick, the same
+                                                 again, form before
                                                  tuning, then each candidate on every level    */
-    int confirm_choice;                       /* index into step_us_confirm of the form kept    */
+    int confirm_choice;                       /* first index into step_us_confirm of the form kept */
     double default_step_us;                   /* coarse step through the graphs before tuning      */
     double step_us[2];                        /* coarse step, chosen kernels, PDL off / on         */
     int pdl;                                  /* chosen: 1 programmatic dependent launch on        */

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <omp.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -1771,7 +1772,12 @@ static lbm_status graph_step_time(lbm_solver *s, int n, double *us)
     return LBM_OK;
 }
 
-static int no_persist(int sched) { return sched == LBM_SCHED_PERSIST ? LBM_SCHED_TILE : sched; }
+static double median_of(std::vector<double> v)
+{
+    std::sort(v.begin(), v.end());
+    const size_t n = v.size();
+    return n % 2 ? v[n / 2] : 0.5 * (v[n / 2 - 1] + v[n / 2]);
+}
 
 lbm_status lbm_autotune(lbm_solver *s, int steps, lbm_tune_report *out)
 {
@@ -1788,8 +1794,9 @@ lbm_status lbm_autotune(lbm_solver *s, int steps, lbm_tune_report *out)
     if ((st = graph_step_time(s, steps, &out->default_step_us)) != LBM_OK) return st;
     int keep_mb[LBM_MAXL], keep_pe[LBM_MAXL], keep_sh[LBM_MAXL];
     for (int l = 0; l < L; l++) { keep_mb[l] = s->min_blocks[l]; keep_pe[l] = s->sched[l]; keep_sh[l] = s->shape[l]; }
-    // 1: register budget and grid schedule per level, from per-launch event timings of
-    //    every candidate
+    // 1: launch form per level, from per-launch event timings of every candidate.  Candidates with
+    //    the same warps per block are the same launches: a form's time is the median of theirs, and
+    //    the first of them stands for it
     for (int c = 0; c < LBM_TUNE_CANDIDATES; c++) {
         for (int l = 0; l < L; l++) { s->min_blocks[l] = CAND_MB[c]; s->sched[l] = CAND_PE[c]; s->shape[l] = CAND_SH[c]; }
         out->candidate_min_blocks[c] = CAND_MB[c];
@@ -1802,38 +1809,58 @@ lbm_status lbm_autotune(lbm_solver *s, int steps, lbm_tune_report *out)
     }
     for (int l = 0; l < L; l++) {
         int best = 0;
-        for (int c = 1; c < LBM_TUNE_CANDIDATES; c++)
-            if (out->level_us[c][l] < out->level_us[best][l]) best = c;
+        double best_us = 0.0;
+        for (int c = 0; c < LBM_TUNE_CANDIDATES; c++) {
+            std::vector<double> us;
+            int first = c;
+            for (int d = LBM_TUNE_CANDIDATES - 1; d >= 0; d--)
+                if (block_warps(CAND_PE[d]) == block_warps(CAND_PE[c])) { us.push_back(out->level_us[d][l]); first = d; }
+            if (first != c) continue;
+            const double m = median_of(us);
+            if (c == 0 || m < best_us) { best_us = m; best = c; }
+        }
         s->min_blocks[l] = CAND_MB[best];
         s->sched[l] = CAND_PE[best];
         s->shape[l] = CAND_SH[best];
-        out->min_blocks[l] = CAND_MB[best];
-        out->sched[l] = CAND_PE[best];
-        out->shape[l] = CAND_SH[best];
     }
-    // 1b: per-launch timings miss how launches overlap inside the graph (a persistent grid
-    //     occupies every SM while the next launch would start): keep the per-level choice
-    //     only if whole graph steps confirm it, against the same choice with one block per
-    //     tile where it took a persistent grid, against the default form, and against each
-    //     candidate on every level
+    // 1b: per-launch timings miss how launches overlap inside the graph: keep the per-level choice
+    //     only if whole graph steps confirm it, against the form before tuning and against each
+    //     candidate on every level, again by the medians of those that are the same launches
     {
         int pick_mb[LBM_MAXL], pick_pe[LBM_MAXL], pick_sh[LBM_MAXL];
         for (int l = 0; l < L; l++) { pick_mb[l] = s->min_blocks[l]; pick_pe[l] = s->sched[l]; pick_sh[l] = s->shape[l]; }
+        const int NV = 3 + LBM_TUNE_CANDIDATES;
         auto form = [&](int v, int l, int &mb, int &pe, int &sh) {
             if (v >= 3) { mb = CAND_MB[v - 3]; pe = CAND_PE[v - 3]; sh = CAND_SH[v - 3]; return; }
             mb = v == 2 ? keep_mb[l] : pick_mb[l];
-            pe = v == 0 ? pick_pe[l] : (v == 1 ? no_persist(pick_pe[l]) : keep_pe[l]);
+            pe = v == 2 ? keep_pe[l] : pick_pe[l];
             sh = v == 2 ? keep_sh[l] : pick_sh[l];
         };
+        auto same = [&](int v, int w) {
+            bool eq = true;
+            for (int l = 0; l < L; l++) {
+                int mb, sh, pv, pw;
+                form(v, l, mb, pv, sh);
+                form(w, l, mb, pw, sh);
+                eq = eq && block_warps(pv) == block_warps(pw);
+            }
+            return eq;
+        };
+        for (int v = 0; v < NV; v++) {
+            for (int l = 0; l < L; l++) form(v, l, s->min_blocks[l], s->sched[l], s->shape[l]);
+            if ((st = capture_graphs(s)) != LBM_OK) return st;
+            if ((st = graph_step_time(s, steps, &out->step_us_confirm[v])) != LBM_OK) return st;
+        }
         double best_us = 0.0;
         int best = 0;
-        for (int v = 0; v < 3 + LBM_TUNE_CANDIDATES; v++) {
-            for (int l = 0; l < L; l++) form(v, l, s->min_blocks[l], s->sched[l], s->shape[l]);
-            double us = 0.0;
-            if ((st = capture_graphs(s)) != LBM_OK) return st;
-            if ((st = graph_step_time(s, steps, &us)) != LBM_OK) return st;
-            out->step_us_confirm[v] = us;
-            if (v == 0 || us < best_us) { best_us = us; best = v; }
+        for (int v = 0; v < NV; v++) {
+            std::vector<double> us;
+            int first = v;
+            for (int w = NV - 1; w >= 0; w--)
+                if (same(v, w)) { us.push_back(out->step_us_confirm[w]); first = w; }
+            if (first != v) continue;
+            const double m = median_of(us);
+            if (v == 0 || m < best_us) { best_us = m; best = v; }
         }
         for (int l = 0; l < L; l++) {
             form(best, l, s->min_blocks[l], s->sched[l], s->shape[l]);
