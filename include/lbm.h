@@ -356,8 +356,8 @@ lbm_status lbm_set_state(lbm_solver *s, const void *buf, size_t size);
 lbm_status lbm_set_launch_variant(lbm_solver *s, const int *min_blocks, const int *sched, const int *shape,
                                   int pdl);
 
-/* The level kernel's work lists of a level in cost order (also on host-only handles; a launch
- * takes the warps in this order, except that plain ones, of active cells only, come last):
+/* The level kernel's work of a level in cost order (also on host-only handles; the list that the
+ * launches run, lbm_get_launch_list, takes the warps in this order with the plain ones last):
  * warps 0 gives the work tiles (tiles holding an active or ghost fluid cell), warps 1 the
  * work warps (the 16 x 2-cell warps w of those tiles, cells x in [16 (w & 1), +16), y in
  * {2 (w >> 1), +1} of the tile, that hold one); both ordered by cost class (a boundary node
@@ -366,6 +366,16 @@ lbm_status lbm_set_launch_variant(lbm_solver *s, const int *min_blocks, const in
  * indices i, j of the tile's first cell and the warp (-1 for tiles); with cap 0 only the
  * count.  Errors: LBM_ERR_INVALID_ARG, LBM_ERR_NO_GEOMETRY. */
 lbm_status lbm_get_work_list(lbm_solver *s, int level, int warps, int *out, int cap, int *n);
+
+/* The list of work warps that the level kernel's launches of a level run (also on host-only
+ * handles), in the order of lbm_get_work_list and its entries: first the warps with a boundary
+ * node of the finest level, each twice in a row (one of the two evaluates the wall function:
+ * n_pair entries), then the other general ones, and last n_plain, an even number, of plain ones:
+ * every cell active fluid without wall, interface or box edge and every tile beside the warp's
+ * cells present.  (With an odd number of those one is among the general ones.)  n_pair and
+ * n_plain may be NULL; with cap 0 only the counts.  Errors: LBM_ERR_INVALID_ARG,
+ * LBM_ERR_NO_GEOMETRY. */
+lbm_status lbm_get_launch_list(lbm_solver *s, int level, int *out, int cap, int *n, int *n_pair, int *n_plain);
 
 /* Load history.  With every > 0, lbm_step and lbm_step_async enqueue, after each coarse step
  * whose count is a multiple of every, what lbm_get_loads computes (the wall state query,

@@ -152,6 +152,7 @@ def _load(path):
         "lbm_get_wall_distance": ([vp, C.c_int, dp, C.c_int], C.c_int),
         "lbm_get_flags": ([vp, C.c_int, C.POINTER(C.c_uint), C.c_int], C.c_int),
         "lbm_get_work_list": ([vp, C.c_int, C.c_int, C.c_void_p, C.c_int, C.POINTER(C.c_int)], C.c_int),
+        "lbm_get_launch_list": ([vp, C.c_int, C.c_void_p, C.c_int, *[C.POINTER(C.c_int)] * 3], C.c_int),
         "lbm_get_prolong_independence": ([vp, C.POINTER(C.c_int), C.c_int], C.c_int),
         "lbm_get_info": ([vp, C.POINTER(lbm_info)], C.c_int),
         "lbm_time_kernels": ([vp, C.c_int, C.POINTER(lbm_kernel_times)], C.c_int),
@@ -433,6 +434,16 @@ class Solver:
         out = np.zeros((max(n.value, 1), 3), dtype=np.int32)
         self._check(self._lib.lbm_get_work_list(self._h, level, w, out.ctypes.data_as(C.c_void_p), n.value, C.byref(n)))
         return out[:n.value]
+
+    def launch_list(self, level):
+        """lbm_get_launch_list: ((n, 3) int array of the work warps that the level kernel runs, as
+        in work_list, n_pair, n_plain)."""
+        n, pair, plain = C.c_int(), C.c_int(), C.c_int()
+        self._check(self._lib.lbm_get_launch_list(self._h, level, None, 0, C.byref(n), C.byref(pair), C.byref(plain)))
+        out = np.zeros((max(n.value, 1), 3), dtype=np.int32)
+        self._check(self._lib.lbm_get_launch_list(self._h, level, out.ctypes.data_as(C.c_void_p), n.value, C.byref(n),
+                                                  None, None))
+        return out[:n.value], pair.value, plain.value
 
     def flags(self, level):
         """The level kernel's 32-bit flag word per cell of the level box."""

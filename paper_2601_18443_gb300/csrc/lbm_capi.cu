@@ -80,6 +80,7 @@ struct HostLevelDev {
     std::vector<int> band_ij;      // global cell indices of the band cells, in band-index order
     std::vector<int> work_tiles;   // host copies of the level kernel's work lists (cost order)
     std::vector<int> work_warps;
+    std::vector<int> launch;       // host copy of v.work, the list the kernel runs
 };
 
 }  // namespace
@@ -882,6 +883,7 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
             v.n_plain = (int)pw.size();
             gw.insert(gw.end(), pw.begin(), pw.end());
             v.work = upload(s, gw, ok);
+            H.launch = std::move(gw);
         }
         v.flags = upload(s, H.flags, ok);
         v.inv_d2 = upload(s, inv_d2, ok);
@@ -1425,6 +1427,26 @@ lbm_status lbm_get_work_list(lbm_solver *s, int level, int warps, int *out, int 
         out[3 * k] = G.tile_x[t] * LBM_TX;
         out[3 * k + 1] = G.tile_y[t] * LBM_TY;
         out[3 * k + 2] = warps ? (w[k] & 7) : -1;
+    }
+    return LBM_OK;
+}
+
+lbm_status lbm_get_launch_list(lbm_solver *s, int level, int *out, int cap, int *n, int *n_pair, int *n_plain)
+{
+    if (!s || !n || (cap > 0 && !out)) return fail(s, LBM_ERR_INVALID_ARG, "bad argument");
+    if (!s->grid_ready) return fail(s, LBM_ERR_NO_GEOMETRY, "no geometry");
+    if (level < 0 || level >= s->L) return fail(s, LBM_ERR_INVALID_ARG, "level out of range");
+    const lbmgrid::Level &G = s->g.lv[level];
+    const std::vector<int> &w = s->lv[level].launch;
+    *n = (int)w.size();
+    if (n_pair) *n_pair = s->lv[level].v.n_pair_warps;
+    if (n_plain) *n_plain = s->lv[level].v.n_plain;
+    if (cap <= 0) return LBM_OK;
+    if ((int)w.size() > cap) return fail(s, LBM_ERR_INVALID_ARG, "capacity too small");
+    for (size_t k = 0; k < w.size(); k++) {
+        out[3 * k] = G.tile_x[w[k] >> 3] * LBM_TX;
+        out[3 * k + 1] = G.tile_y[w[k] >> 3] * LBM_TY;
+        out[3 * k + 2] = w[k] & 7;
     }
     return LBM_OK;
 }
