@@ -96,6 +96,21 @@ struct LevelStep {
     int tl_base;             // record tl_base + blockIdx.x, or null
 };
 
+// Resident blocks of LBM_BLOCK threads per SM that the register allocation of the level kernel must
+// allow (KIND, PLAIN and EDGE of level.cuh).  A launch
+// with plain warps is bound by latency times occupancy, so it runs at 64 registers (32 warps a SM):
+// a 2048^2 level with SA-neg takes 91 us a step at 64 registers, 92 at 72, 98 at 80, a 3008 x 2792
+// laminar one 128, 136 and 145.  Levels with a finer one spill too much there (the explosion):
+// the c/4096 workload's levels 2 and 3 take 5.3 .. 6.4 us at 80 registers and 7.0 .. 8.8 at 64,
+// its level 4 the same at both; its level 0 (box edges) 13.0 / 13.9 us against 13.4 / 15.4 at 80,
+// and the finest one 13.7 / 16.2 against 13.8 / 16.5.  Without plain warps a launch is one general
+// warp's latency: 96 registers, 128 with a finer level, which is no spills (c/256 airfoil 289 us a
+// coarse step against 294 at 80, 260 against 263 with the finer level's target table at 128 and 96).
+__host__ __device__ constexpr int level_min_blocks(int kind, bool plain, bool edge)
+{
+    return plain ? (kind == 1 && !edge ? 6 : 8) : (kind == 1 ? 4 : 5);
+}
+
 // Launch variant of a level's kernels (lbm_set_launch_variant, lbm_autotune): the warps of a
 // block, and whether launches use programmatic dependent launch.
 struct LevelTune {

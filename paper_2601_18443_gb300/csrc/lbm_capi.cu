@@ -333,17 +333,22 @@ static void flush_prolong(lbm_solver *s, cudaStream_t st, long long &nk)
     s->pend_grid = 0;
 }
 
-// Whether a launch over `warps` work warps takes the plain ones two to a warp.  Up to one wave of
-// resident warps (5 blocks of 4 a SM) a launch is one warp's latency, and a warp of one block is
-// the shorter one: 2700 work warps took 4.7 / 5.4 us (even / odd step, the 7-level polar request's
-// finest level) against 5.5 / 6.7 as pairs, 1400 warps 3.0 / 3.8 against 4.8 / 6.0.  Beyond that the
-// work per warp counts: 3100 warps (level 2 of the c/4096 workload) 5.3 / 6.4 us as pairs and
-// 5.4 / 6.3 one by one, 5000 (level 3) 5.5 / 6.3 and 7.6 / 8.4, 8800 (level 4) 8.2 / 10.2 and
-// 11.5 / 13.1.
-static bool plain_form(long warps, int sms) { return warps > 20 * (long)sms; }
-
 // what the level kernel does on a level: 2 finest with wall records, 1 with a finer level, 0 neither
 static int level_kind(const lbm_solver *s, int l) { return l == s->L - 1 ? (s->rec.n > 0 ? 2 : 0) : 1; }
+
+// Whether a launch over `warps` work warps takes the plain ones two to a warp.  Up to one wave of
+// resident warps a launch is one warp's latency, and a warp of one block is the shorter one: 2700
+// work warps took 4.7 / 5.4 us (even / odd step, the 7-level polar request's finest level) against
+// 5.5 / 6.7 as pairs, 1400 warps 3.0 / 3.8 against 4.8 / 6.0.  Beyond that the work per warp counts:
+// 5000 warps (level 3 of the c/4096 workload) 5.5 / 6.3 us as pairs and 7.6 / 8.4 one by one, 8800
+// (level 4) 8.2 / 10.2 and 11.5 / 13.1.  The wave is that of the launch one by one: 20 warps a SM
+// (5 blocks of 4), and 16 with a finer level, whose launches hold more registers.  Between those two
+// lines, 2500 to 2800 warps with a finer level (level 2 of the c/4096 workload with 48 and 52 layers):
+// 5.6 / 6.0 and 5.9 / 6.2 us as pairs, 5.6 / 6.6 and 6.9 / 8.2 one by one.
+static bool plain_form(long warps, int sms, int kind)
+{
+    return warps > (LBM_BLOCK / 32) * (long)lbmdev::level_min_blocks(kind, false, false) * sms;
+}
 
 // warps of a block of the level kernel under a grid schedule
 static int block_warps(int sched) { return sched == LBM_SCHED_WARPS ? 2 : LBM_BLOCK / 32; }
@@ -392,7 +397,7 @@ static void advance(lbm_solver *s, cudaStream_t st, int l, int restrict_up, long
         ls.tl_base = base;
     }
     mark_begin(s);
-    const lbmdev::LevelTune tu{block_warps(s->sched[l]), s->pdl, plain_form(P.n_gen_warps + P.n_plain, s->k.sms)};
+    const lbmdev::LevelTune tu{block_warps(s->sched[l]), s->pdl, plain_form(P.n_gen_warps + P.n_plain, s->k.sms, level_kind(s, l))};
     lbmdev::launch_level(st, P, F, C, s->rec, s->k, ls, tu);
     mark_end(s, l == L - 1 ? KC_LEVEL_FINEST : KC_LEVEL_COARSE, P.ns, l);
     nk++;
@@ -1209,7 +1214,7 @@ lbm_status lbm_step_launch(lbm_solver *s, int level, int kind)
         ls.restrict_up = kind == 1 && C != nullptr;
         ls.pp = C ? s->parity[l - 1] : 0;
             ls.status = s->d_status;
-        const lbmdev::LevelTune tu{block_warps(s->sched[l]), 0, plain_form(P.n_gen_warps + P.n_plain, s->k.sms)};
+        const lbmdev::LevelTune tu{block_warps(s->sched[l]), 0, plain_form(P.n_gen_warps + P.n_plain, s->k.sms, level_kind(s, l))};
         lbmdev::launch_level(s->stream, P, F, C, s->rec, s->k, ls, tu);
         s->parity[l] ^= 1;
     }
@@ -1982,7 +1987,7 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
         else a.edge = a.edge || edge;
         warps += s->lv[l].v.n_gen_warps + s->lv[l].v.n_plain;
     }
-    a.plain = a.kind >= 0 && plain_form(warps, b->m[0]->k.sms);
+    a.plain = a.kind >= 0 && plain_form(warps, b->m[0]->k.sms, a.kind);
     unsigned grid = 0;
     for (lbm_solver *s : b->m) {
         if (l >= s->L) continue;
