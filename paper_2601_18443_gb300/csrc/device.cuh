@@ -14,7 +14,6 @@ namespace lbmdev {
 struct LevelView {
     int ntiles;
     int ns;                       // cell slots = ntiles * 256
-    int n_wall_tiles;             // tiles [0, n_wall_tiles) hold boundary nodes
     const int *tile_x, *tile_y;   // tile coordinates (global, in tiles)
     const int *nbr;               // 9 per tile, D2Q9 order, -1 absent
     const int *child;             // 4 per tile: tiles of level l+1, index b * 2 + a
@@ -44,8 +43,6 @@ struct LevelView {
 // Wall records (finest level), structure of arrays.
 struct RecView {
     int n;
-    const int *bslot;             // slot of the boundary node
-    const int *ns;                // reference stencil size
     const int *st_slot;           // 16 per record
     const float *st_wr;           // 16 per record: inverse-distance weights of rho at R (normalised)
     const float *st_wu;           // 16 per record: weights of u at R (intercept row of the linear LSQ, or the IDW weights)
@@ -86,7 +83,6 @@ struct StepConsts {
 struct LevelStep {
     int p;              // time level of this level (reads [p], writes [p ^ 1]); also the parity of
                         // the in-place population update (0 even, 1 odd)
-    int has_child;      // level l+1 exists
     int is_level0;      // level 0 (box-edge conditions may apply)
     int wall;           // this level holds the wall records (finest level)
     int restrict_up;    // write the restriction of this level's new fields into level l-1

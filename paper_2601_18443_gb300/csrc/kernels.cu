@@ -238,7 +238,6 @@ template <typename T>
 __global__ void k_explode(LevelView P, LevelView F, StepConsts k, const float *post)
 {
     const int t = blockIdx.x, c = threadIdx.x;
-    const int lx = c & 31, ly = c >> 5;
     const int slot = t * LBM_TILE + c;
     const uint32_t fl = P.flags[slot];
     if ((fl & FL_KIND_MASK) != KIND_ACTIVE || (fl & FL_SOLID) || !(fl & FL_BAND)) return;

@@ -382,7 +382,6 @@ static void advance(lbm_solver *s, cudaStream_t st, int l, int restrict_up, long
     flush_prolong(s, st, nk);
     lbmdev::LevelStep ls{};
     ls.p = s->parity[l];
-    ls.has_child = F != nullptr;
     ls.is_level0 = l == 0;
     ls.wall = (l == L - 1) && s->rec.n > 0;
     ls.restrict_up = restrict_up && C != nullptr;
@@ -768,7 +767,6 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         LevelView &v = H.v;
         v.ntiles = G.ntiles;
         v.ns = (int)ns;
-        v.n_wall_tiles = G.n_wall_tiles;
         v.tile_x = upload(s, G.tile_x, ok);
         v.tile_y = upload(s, G.tile_y, ok);
         v.nbr = upload(s, G.nbr, ok);
@@ -913,12 +911,11 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
     const int nr = (int)s->g.recs.size();
     {
         const lbmgrid::Level &G = s->g.lv[L - 1];
-        std::vector<int> bslot(nr), nsv(nr), st_slot((size_t)nr * 16, -1), loop(nr);
+        std::vector<int> bslot(nr), st_slot((size_t)nr * 16, -1), loop(nr);
         std::vector<float> st_wr((size_t)nr * 16, 0.f), st_wu((size_t)nr * 16, 0.f), nx(nr), ny(nr), dwb(nr), q((size_t)nr * 9, 0.f);
         for (int r = 0; r < nr; r++) {
             const lbmgrid::Record &R = s->g.recs[r];
             bslot[r] = (int)G.slot(R.i, R.j);
-            nsv[r] = R.ns;
             double wr[16], wu[16];
             stencil_weights(R, wr, wu);
             for (int m = 0; m < 16; m++) {
@@ -958,8 +955,6 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         }
         RecView &v = s->rec;
         v.n = nr;
-        v.bslot = upload(s, bslot, ok);
-        v.ns = upload(s, nsv, ok);
         v.st_slot = upload(s, st_slot, ok);
         v.st_wr = upload(s, st_wr, ok);
         v.st_wu = upload(s, st_wu, ok);
@@ -1208,12 +1203,11 @@ lbm_status lbm_step_launch(lbm_solver *s, int level, int kind)
         const LevelView *C = (l > 0) ? &s->lv[l - 1].v : nullptr;
         lbmdev::LevelStep ls{};
         ls.p = s->parity[l];
-        ls.has_child = F != nullptr;
         ls.is_level0 = l == 0;
         ls.wall = (l == L - 1) && s->rec.n > 0;
         ls.restrict_up = kind == 1 && C != nullptr;
         ls.pp = C ? s->parity[l - 1] : 0;
-            ls.status = s->d_status;
+        ls.status = s->d_status;
         const lbmdev::LevelTune tu{block_warps(s->sched[l]), 0, plain_form(P.n_gen_warps + P.n_plain, s->k.sms, level_kind(s, l))};
         lbmdev::launch_level(s->stream, P, F, C, s->rec, s->k, ls, tu);
         s->parity[l] ^= 1;
@@ -1999,7 +1993,6 @@ static void batch_advance(lbm_batch *b, cudaStream_t st, int l, int restrict_up,
         d.R = s->rec;
         d.k = s->k;
         d.ls.p = s->parity[l];
-        d.ls.has_child = l + 1 < L;
         d.ls.is_level0 = l == 0;
         d.ls.wall = (l == L - 1) && s->rec.n > 0;
         d.ls.restrict_up = restrict_up && l > 0;

@@ -26,7 +26,6 @@
 
 #include "device.cuh"
 
-
 namespace lbmdev {
 
 // ------------------------------------------------------------------ lattice (eq 2)
@@ -59,16 +58,6 @@ __device__ __forceinline__ void cell_of_thread(int c, int &lx, int &ly)
     const int w = c >> 5, lane = c & 31;
     lx = (w & 1) * 16 + (lane & 15);
     ly = (w >> 1) * 2 + (lane >> 4);
-}
-
-// slot of the cell at offset (dx, dy) from (lx, ly), or -1 if its tile is absent
-__device__ __forceinline__ int nb_slot(const int *nb3, int lx, int ly, int dx, int dy)
-{
-    const int nx = lx + dx, ny = ly + dy;
-    const int sx = nx < 0 ? 0 : (nx >= LBM_TX ? 2 : 1);
-    const int sy = ny < 0 ? 0 : (ny >= LBM_TY ? 2 : 1);
-    const int tt = nb3[sy * 3 + sx];
-    return tt < 0 ? -1 : tt * LBM_TILE + (ny & (LBM_TY - 1)) * LBM_TX + (nx & (LBM_TX - 1));
 }
 
 // The slots of the eight D2Q9 neighbours at offsets +c_q (q = 1..8) and the own slot
@@ -266,12 +255,6 @@ __device__ __forceinline__ void collide_cm(const float g[9], float drho, float j
     o[8] = 0.25f * (-M11 + M21 - M12 + M22);
 }
 
-__device__ __forceinline__ float sa_fv1(float chi)
-{
-    float c3 = chi * chi * chi;
-    return c3 / (c3 + SA_CV1_3);
-}
-
 // 2 - omega for the effective viscosity nu + nu_t (eq 9 with the RANS substitution);
 // the divisions use the fast reciprocal path (about 2 ulp)
 __device__ __forceinline__ float delta_of(float nu, float chi, int turbulence)
@@ -437,7 +420,6 @@ __device__ __forceinline__ float wf_utau(float ut, float y_nu, float guess)
         const float gp = up + yp * wf_dudy(yp);
         if (fabsf(gv) > 0.05f * ut) {
             u *= __powf(__fdividef(ut, u * up), __fdividef(up, gp));
-            if (fabsf(gv) <= 4e-6f * u) break;
             continue;
         }
         const float un = u - __fdividef(gv, gp);
@@ -1363,12 +1345,6 @@ static void launch_pdl_bs(void (*kern)(Args...), unsigned grid, unsigned block, 
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
-template <typename... Args>
-static void launch_pdl(void (*kern)(Args...), unsigned grid, cudaStream_t st, int pdl, Args... args)
-{
-    launch_pdl_bs(kern, grid, LBM_TILE, st, pdl, args...);
 }
 
 // the level holding the wall records is the finest one, which has no child level
