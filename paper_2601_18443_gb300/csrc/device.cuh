@@ -47,7 +47,7 @@ struct RecView {
     const float *st_wr;           // 16 per record: inverse-distance weights of rho at R (normalised)
     const float *st_wu;           // 16 per record: weights of u at R (intercept row of the linear LSQ, or the IDW weights)
     const float *nx, *ny, *dwb;   // unit normal (wall -> fluid), wall distance of B
-    const float *q;               // 9 per record: wall fraction of cut pulled directions
+    const float *v;               // 9 per record: q / (1 + q), q the wall fraction of cut pulled directions
     const int *loop;
     const float *slip;            // prescribed slip per loop (wall model 2), 2 per loop
     float *drhoW, *uWx, *uWy, *utau, *chiB, *tx, *ty, *ut;

@@ -912,7 +912,7 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
     {
         const lbmgrid::Level &G = s->g.lv[L - 1];
         std::vector<int> bslot(nr), st_slot((size_t)nr * 16, -1), loop(nr);
-        std::vector<float> st_wr((size_t)nr * 16, 0.f), st_wu((size_t)nr * 16, 0.f), nx(nr), ny(nr), dwb(nr), q((size_t)nr * 9, 0.f);
+        std::vector<float> st_wr((size_t)nr * 16, 0.f), st_wu((size_t)nr * 16, 0.f), nx(nr), ny(nr), dwb(nr), cut_v((size_t)nr * 9, 0.f);
         for (int r = 0; r < nr; r++) {
             const lbmgrid::Record &R = s->g.recs[r];
             bslot[r] = (int)G.slot(R.i, R.j);
@@ -925,7 +925,7 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
                 st_wu[(size_t)r * 16 + m] = m < R.ns ? (float)wu[m] : 0.f;
             }
             nx[r] = (float)R.n[0]; ny[r] = (float)R.n[1]; dwb[r] = (float)R.dwb;
-            for (int d = 0; d < 9; d++) q[(size_t)r * 9 + d] = (float)R.q[d];
+            for (int d = 0; d < 9; d++) cut_v[(size_t)r * 9 + d] = (float)(R.q[d] / (1.0 + R.q[d]));
             loop[r] = R.loop;
         }
         // per record, the directions q whose node B + c_q is active fluid: its tile is present
@@ -961,7 +961,7 @@ lbm_status lbm_set_geometry(lbm_solver *s, const double *xy, const int *loop_off
         v.nx = upload(s, nx, ok);
         v.ny = upload(s, ny, ok);
         v.dwb = upload(s, dwb, ok);
-        v.q = upload(s, q, ok);
+        v.v = upload(s, cut_v, ok);
         v.loop = upload(s, loop, ok);
         v.nfluid = upload(s, nfluid, ok);
         s->d_slip = (float *)dalloc(s, 2 * (size_t)std::max(n_loops, 1) * sizeof(float));

@@ -746,23 +746,23 @@ __device__ __forceinline__ void pair_wait(int pair)
     else asm volatile("bar.sync 2, 64;" ::: "memory");
 }
 
-// A boundary node's wall fractions and the mask of directions q whose node B + c_q is active
-// fluid (eq 27), read before the wait.
+// A boundary node's weights q / (1 + q) of the wall fractions and the mask of directions q whose node
+// B + c_q is active fluid (eq 27), read before the wait.
 struct CutLinks {
-    float q[9];
+    float v[9];
     uint32_t nf;
 };
 
 // Eq 27 for one cut direction of wall fraction q: gin the population that arrives along the opposite
 // one, fo and f the cell's own last post-collision ones along it and along the direction, mom the
-// wall's momentum term.  ((1 - q) gin + q fo + mom + q f) / (1 + q) = f + (a - f) / (1 + q), so that
-// the roundings of the division and of 1 + q act on the small difference: against 64 bits 2.35e-8
-// rms and 1.6e-7 at most of the populations' size, where weights 1 / (1 + q) and q / (1 + q) rounded
-// to FP32 give 2.66e-8 and 1.8e-7, and the quotient of the whole sum 3.94e-8 and 2.9e-7.
-__device__ __forceinline__ float yu_link(float q, float gin, float fo, float f, float mom)
+// wall's momentum term, v = q / (1 + q).  The quotient ((1 - q) gin + q fo + mom + q f) / (1 + q) is
+// gin + mom + v (fo + f - 2 gin - mom): the roundings act on small differences, and no division
+// follows the wall warp's results.  Error against 64 bits, in the populations' size: 1.4e-8 rms and
+// 0.8e-7 at most; with weights 1 / (1 + q) and q / (1 + q) rounded to FP32 2.7e-8 and 1.8e-7, and
+// dividing the whole sum 3.9e-8 and 2.9e-7.
+__device__ __forceinline__ float yu_link(float v, float gin, float fo, float f, float mom)
 {
-    const float a = (1.0f - q) * gin + q * fo + mom;
-    return f + __fdividef(a - f, 1.0f + q);
+    return gin + (mom + v * ((fo - gin) + (f - gin) - mom));
 }
 
 struct WallStatic {
@@ -976,7 +976,7 @@ __device__ __forceinline__ void general_warp(const LevelView &P, const LevelView
             for (int q = 1; q < 9; q++) {
                 const int qo = oppq(q);
                 const float mom = 6.0f * wq(q) * (1.0f + drW) * (cxq(q) * uWx + cyq(q) * uWy);
-                const float yu = yu_link(cut.q[q], gin[qo], x[qo], x[q], mom);
+                const float yu = yu_link(cut.v[q], gin[qo], x[qo], x[q], mom);
                 const float half = x[qo] + mom;           // half-way form, eq 24
                 if (fl & (1u << (FL_CUT_SHIFT + q - 1))) g[q] = (cut.nf >> q & 1) ? yu : half;
             }
@@ -1227,7 +1227,7 @@ __device__ __forceinline__ CutLinks cut_links(const RecView &R, const GeneralWor
     const int r = b ? checked_index(W.ax, R.n, status) : 0;
     c.nf = b ? __ldg(R.nfluid + r) : 0u;
 #pragma unroll
-    for (int q = 0; q < 9; q++) c.q[q] = b ? __ldg(R.q + r * 9 + q) : 0.0f;
+    for (int q = 0; q < 9; q++) c.v[q] = b ? __ldg(R.v + r * 9 + q) : 0.0f;
     return c;
 }
 

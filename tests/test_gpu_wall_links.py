@@ -2,9 +2,9 @@
 
 Reference for the size of its error: the same equation with the weights 1 / (1 + q) and q / (1 + q)
 rounded from 64 bits to FP32 and every operation rounded to FP32.  The step's form may be no further
-off in the mean square.  The bound on a single value counts its roundings (u = 2^-24): three on the
-way of each term into the first sum, one for the difference, four for the division (2 ulp), two for
-1 + q and the last sum: 10 u times the sum of the terms' magnitudes."""
+off in the mean square.  The bound on a single value counts its roundings (u = 2^-24), with S the sum
+of the terms' magnitudes: one of the weight, four of sums up to 2 S times a weight up to 1/2, the
+product's and two of sums up to 2 S: at most 10 u S."""
 import ctypes as C
 import os
 import subprocess
@@ -53,17 +53,17 @@ def test_a_cut_link_is_as_precise_as_with_tabulated_weights(links, amp, spread):
     n = 1 << 20
     rng = np.random.default_rng(27)
     base = amp * rng.uniform(-1, 1, n)
-    q = rng.uniform(0, 1, n).astype(np.float32)
-    q[:2] = 0.0, 1.0
+    Q = rng.uniform(0, 1, n)
+    Q[:2] = 0.0, 1.0
+    q, wa, wb = (a.astype(np.float32) for a in (Q, 1 / (1 + Q), Q / (1 + Q)))
     gin, fo, f = ((base + spread * amp * rng.uniform(-0.5, 0.5, n)).astype(np.float32) for _ in range(3))
     mom = (0.3 * amp * rng.uniform(-0.5, 0.5, n)).astype(np.float32)
-    v = np.ascontiguousarray(np.stack([q, gin, fo, f, mom]))
+    v = np.ascontiguousarray(np.stack([wb, gin, fo, f, mom]))
     out = np.empty(n, dtype=np.float32)
     ptr = lambda a: a.ctypes.data_as(C.c_void_p)
     assert links(ptr(v), ptr(out), n) == 0
-    Q, G, Fo, F, M = (a.astype(np.float64) for a in v)
+    G, Fo, F, M = (a.astype(np.float64) for a in v[1:])
     want = ((1 - Q) * G + Q * Fo + M + Q * F) / (1 + Q)
-    wa, wb = (1 / (1 + Q)).astype(np.float32), (Q / (1 + Q)).astype(np.float32)
     table = ((np.float32(1) - q) * gin + q * fo + mom) * wa + wb * f
     rms = lambda x: np.sqrt(np.mean((x.astype(np.float64) - want) ** 2))
     assert rms(out) <= rms(table), (rms(out), rms(table))
