@@ -308,8 +308,8 @@ lbm_status lbm_time_kernels(lbm_solver *s, int n_coarse_steps, lbm_kernel_times 
  * the first of them in the report.
  * Then it picks whether launches use programmatic dependent launch, from the time
  * of `steps` coarse steps through the step graphs each way, and recaptures the graphs with
- * the choice.  The variants compute the same numbers up to FP32 rounding (the compiler
- * schedules and contracts the arithmetic differently per variant); the timed steps are real
+ * the choice.  The forms run the same code in blocks of two or four warps and compute the same
+ * numbers; the timed steps are real
  * steps of the solve (steps_taken of them).
  * Synchronous.  Errors as lbm_step. */
 #define LBM_TUNE_CANDIDATES 12

@@ -1071,9 +1071,9 @@ __device__ __forceinline__ void row4(const float *a, int left, int mid, int righ
 // One warp over two plain 16 x 2-cell blocks (every cell active, none with a wall, interface or
 // box edge, all neighbour tiles present), sixteen lanes a block, two cells of a row a lane.  No
 // flag word is read and nothing branches on a cell.  Fields and populations move as pairs, and a
-// stencil row costs two more scalar loads instead of four: 350 instructions a cell with SA-neg
-// where one cell a lane took 640 (even) and 750 (odd).  The populations come through the thread's
-// own shared memory (buf, asynchronous copies): they are in flight during the SA-neg update
+// stencil row costs two more scalar loads instead of four: 422 (even) and 446 (odd) warp instructions
+// for 32 cells with SA-neg where one cell a lane took 641 and 751.  The populations come through the
+// thread's own shared memory (buf, asynchronous copies): they are in flight during the SA-neg update
 // without holding registers, so one round of memory latency is exposed instead of two.
 // 2048^2 level, SA-neg, FP32: 126.5 -> 91 us a step (5.0 TB/s of the method's 108 B a cell); 3008 x
 // 2792, laminar: 185 -> 128 us (5.8 TB/s of 88 B); 1536 x 2048, SA-neg, BF16: 100 -> 66.6 us.
